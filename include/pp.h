@@ -125,7 +125,8 @@ typedef enum {
 enum {
     PP_OPT_ACC = 1,            /* value: a pp_acc                                              */
     PP_OPT_STREAM = 2,         /* value: cudaStream_t cast to int64 (0 = the context's own)   */
-    PP_OPT_SPLIT = 3,          /* value: j-split count S >= 1, or 0 for automatic              */
+    PP_OPT_SPLIT = 3,          /* value: j-split count S >= 1 (pair-symmetric kernels: ranges a
+                                  row of tiles is cut into), or 0 for automatic              */
     PP_OPT_GRAPH_BLOCK = 4,    /* value: steps per captured CUDA graph (0 = plain launches)   */
     PP_OPT_TIMEOUT_NS = 5,     /* value: limit of each device-side wait in ns (default 1e9, or
                                   the environment variable PP_TIMEOUT_NS at creation)        */
@@ -175,10 +176,12 @@ typedef enum {
  * Create a context for N macro-electrons of common weight w (Sec. 2.1 assumes
  * one weight for all macro-particles), time step dt > 0 and softening
  * eps >= 0 (metres).  Allocates the state and staging buffers on the current
- * CUDA device; force passes allocate their workspaces on first use (the j-split
- * partial sums; with guarded staging from N = 98304 on, the spatial-order
- * workspace, 44 to 52 bytes per particle) and return PP_ERR_NOMEM if that
- * fails.  N >= 1 (N = 0 -> PP_ERR_ARG); N <= 2^28.  On success *out receives
+ * CUDA device; force passes allocate their workspaces on first use (the partial
+ * sums, 1 to 5 KB per particle where the pair-symmetric kernels run, which is by
+ * default from about N = 15000 to 2^22; with guarded staging from N = 98304 on,
+ * the spatial-order workspace, 44 to 52 bytes per particle) and return
+ * PP_ERR_NOMEM if that fails; without room for the partial sums of the symmetric
+ * kernels a context goes on with the one-sided ones.  N >= 1 (N = 0 -> PP_ERR_ARG); N <= 2^28.  On success *out receives
  * the context; on failure *out is set to NULL.
  */
 pp_status pp_create(int64_t N, double w, double dt, double softening, pp_ctx **out);
@@ -433,7 +436,9 @@ const char *pp_last_error(const pp_ctx *ctx);
  * tuning tools), or NULL past the last one.  Names read
  * "<pairs>.<fold>.t<threads>r<targets per thread>k<tile>", e.g.
  * "f32x2.fold64.t256r4k256": packed FP32x2 pair math, FP64 fold, 256 threads,
- * 4 targets per thread, 256-source tiles.
+ * 4 targets per thread, 256-source tiles; or "<pairs>.<fold>.sym<packs>k<tile>"
+ * for the pair-symmetric kernels (each unordered pair evaluated once), `packs`
+ * pairs of targets per thread.
  */
 const char *pp_variant_name(int index);
 

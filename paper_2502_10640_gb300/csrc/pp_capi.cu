@@ -74,6 +74,19 @@ struct pp_ctx {
     unsigned *res_flags = nullptr; // grid-barrier counter of the resident kernel
     void *ord_ws = nullptr;        // spatial-order workspace (tile-box guard variants)
     size_t ord_bytes = 0;
+    // pair-symmetric passes: the plans made so far (an AUTO decision runs several
+    // variants) and the partial sums they share
+    struct SymEntry {
+        std::pair<int, int> key;   // (variant, split)
+        void *tab;                 // items, rows, queue words
+        SymArgs args;              // jrow and ipart are set per launch
+        size_t row_doubles;
+        int grid;
+    };
+    std::vector<SymEntry> sym;
+    double *sym_ws = nullptr;
+    size_t sym_ws_bytes = 0;
+    bool sym_off = false;          // the partial sums could not be allocated
     double *mom_host = nullptr;    // pinned
     int *err_host = nullptr;       // pinned copy of err[0..1], read after each synchronisation
 
@@ -137,6 +150,58 @@ const Variant *variant_by_name(const char *want)
 constexpr int64_t kBoxGuardMinN = 98304;
 constexpr int64_t kBoxGuardWideN = 196608;
 
+// The pair-symmetric kernel (each unordered pair once, pp_sym.cuh) for this
+// context's modes and N, or null where the one-sided kernels are faster.  Its
+// smallest unit of work is a warp's 256 or 512 targets against one tile, so
+// small N leaves too few units; from there on it runs 14 FP32 lane operations
+// per unordered pair instead of 22.  The lines lie where the GB300 sweep has the
+// two level (ms per step, symmetric against one-sided, single staging: 0.104
+// against 0.128 at N = 16384, 0.196 / 0.238 at 24576, 0.315 / 0.407 at 32768,
+// 1.16 / 1.47 at 65536, 4.37 / 5.79 at 131072, 16.8 / 22.5 at 262144; guarded
+// 0.239 / 0.264 at 24576, 1.29 / 1.67 at 65536; on sorted sources 4.64 / 6.13 at
+// 131072, 283 / 366 at 2^20; hi/lo 0.146 / 0.200 at 16384, 27.4 / 33.4 at 262144; weights 0.128 /
+// 0.139 at 16384, 21.2 / 24.3 at 262144).  Tiles of 128 sources below 28672
+// and 256 (512 for single staging) from 196608 on keep the FP32 partial sums no
+// longer than those of the one-sided kernel that would run instead.  Above 2^22
+// the partial sums would pass 18 GB for a step of seconds: one-sided again.
+constexpr int64_t kSymMaxN = int64_t(1) << 22;
+const Variant *sym_variant(const pp_ctx *c)
+{
+    const int64_t n = c->n;
+    const bool kahan = c->acc == PP_ACC_KAHAN;
+    if (c->sym_off || n > kSymMaxN) return nullptr;
+    if (c->positions == PP_POS_SPLIT) {
+        if (n < 13000) return nullptr;
+        return variant_by_name(c->wts ? "f32x2wsplit.fold64.sym4k128"
+                               : kahan ? "f32x2split.kahan.sym4k128"
+                                       : "f32x2split.fold64.sym4k128");
+    }
+    if (c->positions == PP_POS_GUARDED) {
+        if (n < 20000) return nullptr;
+        if (c->wts)
+            return variant_by_name(n >= kBoxGuardMinN ? "f32x2wbguard.sfold64.sym8k256"
+                                                      : "f32x2wguard.fold64.sym4k128");
+        if (kahan)
+            return variant_by_name(n >= kBoxGuardWideN ? "f32x2bguard.kahan.sym8k256"
+                                   : n >= 36864        ? "f32x2guard.kahan.sym8k128"
+                                                       : "f32x2guard.kahan.sym4k128");
+        return variant_by_name(n >= kBoxGuardWideN  ? "f32x2bguard.sfold64.sym8k256"
+                               : n >= kBoxGuardMinN ? "f32x2bguard.sfold64.sym8k128"
+                               : n >= 36864         ? "f32x2guard.fold64.sym8k128"
+                                                    : "f32x2guard.fold64.sym4k128");
+    }
+    if (n < (c->wts ? 15360 : 14336)) return nullptr;
+    if (c->wts)
+        return variant_by_name(n >= 28672 ? "f32x2w.fold64.sym8k256" : "f32x2w.fold64.sym4k128");
+    if (kahan)
+        return variant_by_name(n >= 28672 ? "f32x2.kahan.sym8k256" : "f32x2.kahan.sym4k128");
+    return variant_by_name(n >= 196608  ? "f32x2.fold64.sym8k512"
+                           : n >= 28672 ? "f32x2.fold64.sym8k256"
+                                        : "f32x2.fold64.sym4k128");
+}
+
+const Variant *one_sided_variant(const pp_ctx *c);
+
 // The variant that runs this context's force passes: the override if it fits
 // the accumulation and positions modes, else the default for N.
 const Variant *force_variant(const pp_ctx *c)
@@ -149,6 +214,14 @@ const Variant *force_variant(const pp_ctx *c)
         const Variant &v = vs[c->variant_override];
         if (v.kind == want_kind && v.acc == c->acc && v.positions == c->positions) return &v;
     }
+    const Variant *sym = sym_variant(c);
+    return sym ? sym : one_sided_variant(c);
+}
+
+// The one-sided default for N (FP32 pair paths), with the same staging layout as
+// the symmetric one.
+const Variant *one_sided_variant(const pp_ctx *c)
+{
     const bool big = c->n >= 32768, mid = c->n >= 8192;
     if (c->positions == PP_POS_GUARDED) {   // hi/lo staged, hi parts streamed
         if (c->wts)
@@ -276,13 +349,20 @@ struct Plan {
 
 // Choose S, the number of j-chunks per i-block, to fill the GPU: minimise
 // (waves of CTAs) x (tiles per CTA + fixed per-CTA overhead).
-Plan make_plan(pp_ctx *c, int kind)
+Plan make_plan(pp_ctx *c, int kind, bool one_sided = false)
 {
     Plan pl{};
     pl.v = pick_variant(c, kind);
+    if (one_sided && pl.v->sym) pl.v = one_sided_variant(c);
     const int BI = pl.v->T * pl.v->R;
     pl.nib = (int)((c->n + BI - 1) / BI);
     pl.nipad = pl.nib * BI;
+    if (pl.v->sym) {   // the work items are cut by ensure_sym
+        pl.nsplit = 1;
+        pl.jchunk = c->npad;
+        pl.grid = 0;
+        return pl;
+    }
     const int tiles = c->npad / pl.v->tile;
     const int occ = resident_ctas(*pl.v);
     const int64_t slots = (int64_t)c->sms * occ;
@@ -319,8 +399,79 @@ Plan make_plan(pp_ctx *c, int kind)
     return pl;
 }
 
+// A context keeps this many pair-symmetric plans (the oldest goes first).
+constexpr size_t kSymPlans = 8;
+
+// Device tables and partial sums of a pair-symmetric pass, made once per
+// (variant, split) of the context.  *at: its place in c->sym.
+pp_status ensure_sym(pp_ctx *c, const Variant &v, int *at)
+{
+    int count = 0;
+    const std::pair<int, int> key{(int)(&v - variants(&count)), c->split_override};
+    for (size_t k = 0; k < c->sym.size(); ++k)
+        if (c->sym[k].key == key) {
+            *at = (int)k;
+            return PP_OK;
+        }
+    const int64_t slots = (int64_t)c->sms * resident_ctas(v);
+    const SymPlan sp = make_sym_plan((int)c->n, c->npad, v.R / 2, slots, c->split_override);
+    const size_t ib = round_up(sp.items.size() * sizeof(SymItem), 256);
+    const size_t rb = round_up(sp.rows.size() * sizeof(int2), 256);
+    const size_t ws = (sp.row_doubles + sp.part_doubles) * sizeof(double);
+    // a pass with the old buffers may be running, or captured in a graph
+    if (ws > c->sym_ws_bytes || c->sym.size() >= kSymPlans) {
+        drop_graphs(c);
+        PP_CUDA(cudaStreamSynchronize(c->stream));
+    }
+    if (c->sym.size() >= kSymPlans) {
+        cudaFree(c->sym.front().tab);
+        c->sym.erase(c->sym.begin());
+    }
+    if (ws > c->sym_ws_bytes) {
+        cudaFree(c->sym_ws);
+        c->sym_ws = nullptr;
+        c->sym_ws_bytes = 0;
+        if (cudaMalloc(&c->sym_ws, ws) != cudaSuccess) {
+            cudaGetLastError();
+            return fail(PP_ERR_NOMEM, "cannot allocate the partial sums of the symmetric pass");
+        }
+        c->sym_ws_bytes = ws;
+    }
+    pp_ctx::SymEntry e{};
+    e.key = key;
+    if (cudaMalloc(&e.tab, ib + rb + 256) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(PP_ERR_NOMEM, "cannot allocate the work-item tables");
+    }
+    unsigned char *t = static_cast<unsigned char *>(e.tab);
+    if (cudaMemcpyAsync(t, sp.items.data(), sp.items.size() * sizeof(SymItem),
+                        cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
+        cudaMemcpyAsync(t + ib, sp.rows.data(), sp.rows.size() * sizeof(int2),
+                        cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
+        cudaMemsetAsync(t + ib + rb, 0, 256, c->stream) != cudaSuccess ||
+        cudaStreamSynchronize(c->stream) != cudaSuccess) {   // the host tables end with this call
+        cudaFree(e.tab);
+        return cuda_fail(cudaGetLastError(), "work-item tables");
+    }
+    e.args.items = reinterpret_cast<const SymItem *>(t);
+    e.args.rows = reinterpret_cast<const int2 *>(t + ib);
+    e.args.ctl = reinterpret_cast<unsigned *>(t + ib + rb);
+    e.args.nitems = (int)sp.items.size();
+    e.args.ki = sp.ki;
+    e.row_doubles = sp.row_doubles;
+    // the particles are shared out 32 to a CTA, so a few items do not mean a small grid
+    e.grid = (int)std::min<int64_t>(slots, std::max<int64_t>((sp.items.size() + 3) / 4,
+                                                             (c->n + 31) / 32));
+    c->sym.push_back(e);
+    *at = (int)c->sym.size() - 1;
+    return PP_OK;
+}
+
 pp_status ensure_workspace(pp_ctx *c, const Plan &pl)
 {
+    int at = 0;
+    if (pl.v->sym)
+        if (pp_status st = ensure_sym(c, *pl.v, &at)) return st;
     if (pl.v->order) {
         const size_t need = order_workspace_bytes(c->npad, pl.v->tile);
         if (need > c->ord_bytes) {
@@ -336,6 +487,7 @@ pp_status ensure_workspace(pp_ctx *c, const Plan &pl)
         }
     }
     const int ncomp = (pl.v->kind == KIND_PHI32) ? 1 : 3;
+    if (pl.v->sym) return PP_OK;
     const size_t need = (pl.nsplit > 1 && pl.v->cluster == 0)
                             ? (size_t)pl.nsplit * ncomp * pl.nipad * sizeof(double)
                             : 0;
@@ -437,15 +589,40 @@ cudaError_t launch_force(pp_ctx *c, const Plan &pl, ForceArgs a)
         a.perm = w.perm;
         a.boxes = w.boxes;
     }
+    if (pl.v->sym) {
+        int at = 0;
+        if (ensure_sym(c, *pl.v, &at) != PP_OK) return cudaErrorMemoryAllocation;   // made already
+        SymArgs q = c->sym[at].args;
+        q.jrow = c->sym_ws;
+        q.ipart = c->sym_ws + c->sym[at].row_doubles;
+        return launch_sym(*pl.v, a, q, c->sym[at].grid, c->stream);
+    }
     return launch_variant(*pl.v, a, pl.grid, c->stream);
+}
+
+// The plan of a pass with its workspaces.  Where the default plan is symmetric
+// and its partial sums cannot be allocated, the context goes on with the
+// one-sided kernels.
+pp_status plan_pass(pp_ctx *c, int kind, bool one_sided, Plan *pl)
+{
+    *pl = make_plan(c, kind, one_sided);
+    pp_status st = ensure_workspace(c, *pl);
+    if (st == PP_ERR_NOMEM && pl->v->sym && pl->v == sym_variant(c)) {
+        c->sym_off = true;
+        drop_graphs(c);
+        *pl = make_plan(c, kind, one_sided);
+        st = ensure_workspace(c, *pl);
+    }
+    return st;
 }
 
 // One force pass over staged sources src.
 pp_status force_pass(pp_ctx *c, int mode, const void *src, void *dst, double *out)
 {
     const int kind = (mode == MODE_PHI) ? KIND_PHI32 : (f64_pairs(c) ? KIND_FORCE64 : KIND_FORCE32);
-    const Plan pl = make_plan(c, kind);
-    pp_status st = ensure_workspace(c, pl);
+    // the symmetric kernels make no tile copies: the test hook takes a one-sided one
+    Plan pl{};
+    pp_status st = plan_pass(c, kind, c->skip_copy != 0, &pl);
     if (st != PP_OK) return st;
     ForceArgs a = base_args(c, pl, mode, src, dst, out);
     a.skip_copy = c->skip_copy;
@@ -648,8 +825,8 @@ pp_status build_graphs(pp_ctx *c)
 {
     drop_graphs(c);
     const int kind = f64_pairs(c) ? KIND_FORCE64 : KIND_FORCE32;
-    const Plan pl = make_plan(c, kind);
-    pp_status st = ensure_workspace(c, pl);
+    Plan pl{};
+    pp_status st = plan_pass(c, kind, false, &pl);
     if (st != PP_OK) return st;
     for (int p0 = 0; p0 < 2; ++p0) {
         cudaGraph_t g = nullptr;
@@ -926,6 +1103,8 @@ pp_status pp_destroy(pp_ctx *c)
     cudaFree(c->err);
     cudaFree(c->res_flags);
     cudaFree(c->ord_ws);
+    for (auto &e : c->sym) cudaFree(e.tab);
+    cudaFree(c->sym_ws);
     if (c->mom_host) cudaFreeHost(c->mom_host);
     if (c->err_host) cudaFreeHost(c->err_host);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
@@ -1448,7 +1627,8 @@ pp_status pp_autotune(pp_ctx *c, pp_tune_result *out)
         int cand[4] = {base.nsplit, std::max(1, base.nsplit / 2), std::min(tiles, 2 * base.nsplit),
                        std::max(1, base.nsplit / 4)};
         st = stage_current(c, scratch, vs[v].stage);
-        const int ncand = vs[v].cluster > 0 ? 1 : 4;   // a cluster fixes the split
+        if (vs[v].sym) cand[0] = 0;                    // the plan's own ranges
+        const int ncand = vs[v].cluster > 0 || vs[v].sym ? 1 : 4;   // a cluster fixes the split
         for (int k = 0; k < ncand && st == PP_OK; ++k) {
             bool dup = false;
             for (int q = 0; q < k; ++q) dup |= cand[q] == cand[k];

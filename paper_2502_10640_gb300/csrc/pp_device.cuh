@@ -108,6 +108,14 @@ __device__ __forceinline__ float rsqrt_sfu(float x)
     return y;
 }
 
+// Hardware (SFU) approximate reciprocal, denormals flushed.
+__device__ __forceinline__ float rcp_sfu(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // ---- thread-block clusters (distributed shared memory) ----
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
@@ -143,6 +151,14 @@ __device__ __forceinline__ int ld_peer_s32(uint32_t addr)
 {
     int v;
     asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+    return v;
+}
+
+// Acquire load of a counter that other CTAs of this launch advance.
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *p)
+{
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 

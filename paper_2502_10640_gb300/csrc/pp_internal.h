@@ -8,10 +8,12 @@
 #include <mutex>
 #include <set>
 #include <utility>
+#include <vector>
 
 #include <nvtx3/nvToolsExt.h>
 
 #include "pp_force.cuh"
+#include "pp_sym.cuh"
 
 namespace ppk {
 
@@ -49,6 +51,7 @@ struct Variant {
                   // global-partial chunks chosen by the planner, else exactly `cluster`)
     int positions;  // PosKind
     int order = 0;  // 1: the pass sorts the staged sources in space first (tile-box guard)
+    int sym = 0;    // 1: each unordered pair once (pp_sym.cuh); R targets per thread, `tile` sources
 };
 
 // One-time set-up per (device, key), e.g. a kernel's shared-memory attribute:
@@ -83,6 +86,22 @@ void set_last_error(const char *msg);
 
 // Table of compiled force-kernel variants.
 const Variant *variants(int *count);
+
+// Pair-symmetric kernels (pp_sym.cu): their table entries, the work plan of one
+// pass (host arrays; the caller keeps device copies) and the launcher.
+// Partial-sum rows: at most this many groups of target blocks, so the rows take
+// at most 12 * kSymMaxRows bytes per particle.
+constexpr int kSymMaxRows = 128;
+struct SymPlan {
+    int ki = 1;
+    std::vector<SymItem> items;
+    std::vector<int2> rows;
+    size_t row_doubles = 0, part_doubles = 0;
+};
+std::vector<Variant> sym_variants();
+SymPlan make_sym_plan(int n, int npad, int pk, int64_t slots, int split);
+cudaError_t launch_sym(const Variant &v, const ForceArgs &a, const SymArgs &q, int grid,
+                       cudaStream_t stream);
 
 // Launch one variant with the given arguments on `stream`.
 cudaError_t launch_variant(const Variant &v, const ForceArgs &a, int grid, cudaStream_t stream);

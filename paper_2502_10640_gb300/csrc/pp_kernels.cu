@@ -1,6 +1,7 @@
 // pp_kernels.cu -- the table of compiled force-kernel variants and their launcher.
 #include <cfloat>
 #include <cmath>
+#include <iterator>
 
 #include "pp_internal.h"
 
@@ -157,14 +158,20 @@ const Variant kVariants[] = {
 
 const Variant *variants(int *count)
 {
-    *count = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
-    return kVariants;
+    static const std::vector<Variant> all = [] {
+        std::vector<Variant> v(std::begin(kVariants), std::end(kVariants));
+        for (const Variant &s : sym_variants()) v.push_back(s);
+        return v;
+    }();
+    *count = (int)all.size();
+    return all.data();
 }
 
 cudaError_t launch_variant(const Variant &v, const ForceArgs &a, int grid, cudaStream_t stream)
 {
     static DeviceOnce smem_attr, cluster_attr;
-    const int idx = (int)(&v - kVariants);
+    int count = 0;
+    const int idx = (int)(&v - variants(&count));
     cudaError_t e = smem_attr.run(idx, [&] {
         return cudaFuncSetAttribute(v.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)v.smem);
     });
