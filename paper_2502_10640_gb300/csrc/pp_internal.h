@@ -99,7 +99,7 @@ struct SymPlan {
     size_t row_doubles = 0, part_doubles = 0;
 };
 std::vector<Variant> sym_variants();
-SymPlan make_sym_plan(int n, int npad, int pk, int64_t slots, int split);
+SymPlan make_sym_plan(int n, int npad, const Variant &v, int64_t slots, int split);
 cudaError_t launch_sym(const Variant &v, const ForceArgs &a, const SymArgs &q, int grid,
                        cudaStream_t stream);
 

@@ -3,7 +3,7 @@
 #include <algorithm>
 
 #include "pp_internal.h"
-#include "pp_sym.cuh"
+#include "pp_sym64.cuh"
 
 namespace ppk {
 
@@ -17,6 +17,16 @@ Variant make_sym(const char *name)
               reinterpret_cast<const void *>(
                   &force_sym_kernel<PK, TJ, POS, BOX, WEIGHTED, KAHAN, MINB, RCP>),
               kSymWarps * sym_warp_smem<PK, TJ>(), 0, POS, BOX ? 1 : 0};
+    v.sym = 1;
+    return v;
+}
+
+template <bool WEIGHTED>
+Variant make_sym64(const char *name)
+{
+    Variant v{name, KIND_FORCE64, ACC_FP64FULL, STAGE_F64, kSymThreads,
+              kSym64Targets / 32, kSym64Unit, 0,
+              reinterpret_cast<const void *>(&force_sym64_kernel<WEIGHTED>), 0, 0, POS_SINGLE};
     v.sym = 1;
     return v;
 }
@@ -52,6 +62,8 @@ std::vector<Variant> sym_variants()
         S("f32x2wbguard.sfold64.sym8k256", 8, 256, POS_GUARDED, true, false, 2, 1, true),
         S("f32x2wsplit.fold64.sym4k128", 4, 128, POS_SPLIT, true, false, 3, 0),
 #undef S
+        make_sym64<false>("f64.full.symr1k32"),
+        make_sym64<true>("f64w.full.symr1k32"),
     };
 }
 
@@ -65,10 +77,11 @@ std::vector<Variant> sym_variants()
 // 0.196 at 24576, 0.339 / 0.315 at 32768, 1.16 / 1.17 at 65536).  split > 0 cuts
 // every row into npad / split.  Each item keeps its own sums, which bounds how
 // finely the work may be cut: rows and items take 5 KB per particle at 2^20.
-SymPlan make_sym_plan(int n, int npad, int pk, int64_t slots, int split)
+SymPlan make_sym_plan(int n, int npad, const Variant &v, int64_t slots, int split)
 {
     SymPlan pl;
-    const int WI = 64 * pk, BU = WI / kSymUnit, nu = npad / kSymUnit;
+    const bool f64 = v.kind == KIND_FORCE64;
+    const int WI = 32 * v.R, unit = f64 ? kSym64Unit : kSymUnit, BU = WI / unit, nu = npad / unit;
     const int nib = (n + WI - 1) / WI;
     // the rows of partial sums take 24 bytes x npad x groups / 2
     pl.ki = std::max(1, (nib + kSymMaxRows - 1) / kSymMaxRows);
@@ -77,7 +90,7 @@ SymPlan make_sym_plan(int n, int npad, int pk, int64_t slots, int split)
     for (int g = 0; g < groups; ++g)
         left += (double)std::min(pl.ki, nib - g * pl.ki) * (nu - g * pl.ki * BU);
     const double warps = kSymWarps * (double)slots, most = left / (4.0 * warps);
-    const int least = n >= 20480 && n < 40960 ? 4 : 2;
+    const int least = f64 ? 1 : n >= 20480 && n < 40960 ? 4 : 2;
     for (int g = 0; g < groups; ++g) {
         const int ib0 = g * pl.ki, nb = std::min(pl.ki, nib - ib0);
         const int first = (int)pl.items.size();
@@ -85,7 +98,7 @@ SymPlan make_sym_plan(int n, int npad, int pk, int64_t slots, int split)
             int len = split > 0 ? (nu + split - 1) / split
                                 : (int)(std::min(left / (2.0 * warps), most) / nb);
             len = std::max(1, std::min(std::max(len, split > 0 ? 1 : least), nu - u));
-            pl.items.push_back(SymItem{ib0, nb, u * kSymUnit, (u + len) * kSymUnit});
+            pl.items.push_back(SymItem{ib0, nb, u * unit, (u + len) * unit});
             left -= (double)nb * len;
             u += len;
         }

@@ -241,11 +241,11 @@ __device__ __noinline__ void sym_slow(const float *__restrict__ src, size_t lo_a
 // additions is fixed by the plan: the rows of the groups up to the particles'
 // own, then the items of that group, eight at a time, the chunks of eight dealt
 // to the four warps, whose sums are added in warp order.
-template <int PK, int KIND>
+template <int WI, int KIND>
 __device__ __forceinline__ void sym_finish(const ForceArgs &p, const SymArgs &q, int j0,
                                            double *scratch)
 {
-    constexpr int WI = 64 * PK, U = 8;
+    constexpr int U = 8;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int bis = WI * q.ki;
     const int ib = j0 / WI, grp = ib / q.ki;
@@ -284,12 +284,52 @@ __device__ __forceinline__ void sym_finish(const ForceArgs &p, const SymArgs &q,
     }
 }
 
+// The end of a pass, for every warp after its last item (`done`: items it ran):
+// count them, wait until all items of the pass are done, share out the
+// particles.  scratch: 768 doubles of shared memory.
+template <int WI, int KIND>
+__device__ __forceinline__ void sym_collect(const ForceArgs &p, const SymArgs &q, int done,
+                                            double *scratch, int *s_next)
+{
+    const int tid = threadIdx.x, lane = tid & 31;
+    __threadfence();   // the sums before the count
+    __syncwarp();
+    if (lane == 0) atomicAdd(&q.ctl[SYM_DONE], (unsigned)done);
+
+    // Every item has been handed out, each to a warp that runs now: wait (bounded, by at
+    // least a second: it covers the other warps' last items) until all are done, then
+    // share out the particles.
+    __syncthreads();
+    if (tid == 0) {
+        int ok = 1;
+        const uint64_t t0 = globaltimer_ns();
+        const uint64_t limit = p.timeout_ns > 1000000000ull ? p.timeout_ns : 1000000000ull;
+        while (ld_acquire(&q.ctl[SYM_DONE]) < (unsigned)q.nitems)
+            if (globaltimer_ns() - t0 > limit) {
+                ok = 0;
+                break;
+            }
+        if (!ok) atomicOr(p.err, 1);
+        s_next[0] = ok ? (int)atomicAdd(&q.ctl[SYM_FINISH], 1u) : (1 << 26) - 1;
+    }
+    __syncthreads();
+    __threadfence();
+    int unit = s_next[0];
+    for (int turn = 1; unit * 32 < p.n; turn ^= 1) {
+        if (tid == 0) s_next[turn] = (int)atomicAdd(&q.ctl[SYM_FINISH], 1u);
+        sym_finish<WI, KIND>(p, q, unit * 32, scratch + turn * 384);
+        unit = s_next[turn];
+    }
+    if (tid == 0 && atomicAdd(&q.ctl[SYM_LEFT], 1u) == gridDim.x - 1)
+        for (int k = 0; k < SYM_CTL; ++k) q.ctl[k] = 0u;
+}
+
 // One (warp, tile): the fast pair loop over the 64 PK targets from i0 and the
-// `count` <= TJ sources from j0 (a multiple of 32), then the fold into acc (from place at0 of WI).  Without OWN
-// the sources' sums go to `stash` ([3][TJ] of this warp; ADD: onto what is
-// there), every four steps, so that an FP32 partial holds 8 PK terms.  OWN: the
-// sources are among the targets; each target takes its sum only (the pair comes
-// again with the roles exchanged) and skips itself by index.  Returns false (for
+// `count` <= TJ sources from j0 (a multiple of 32), then the fold into acc (from
+// place at0 of WI).  Without OWN the sources' sums go to `stash` ([3][TJ] of this
+// warp; ADD: onto what is there), every four steps, so that an FP32 partial holds
+// 8 PK terms.  OWN: the sources are among the targets; each target takes its sum
+// only (the pair comes again with the roles exchanged) and skips itself by index.  Returns false (for
 // the whole warp, nothing folded, stash void) for a tile with a zero-distance
 // pair (non-finite sum) or, with POS_GUARDED, with a pair too close for the hi
 // parts alone.  BOX: the caller has ruled close pairs out.  Not inlined: the loop needs every register for
@@ -605,37 +645,8 @@ __global__ void __launch_bounds__(kSymThreads, MINB)
             __syncwarp();
         }
     }
-    __threadfence();   // the sums before the count
-    __syncwarp();
-    if (lane == 0) atomicAdd(&q.ctl[SYM_DONE], (unsigned)done);
-
-    // Every item has been handed out, each to a warp that runs now: wait (bounded, by at
-    // least a second: it covers the other warps' last items) until all are done, then
-    // share out the particles.
-    __syncthreads();
-    if (tid == 0) {
-        int ok = 1;
-        const uint64_t t0 = globaltimer_ns();
-        const uint64_t limit = p.timeout_ns > 1000000000ull ? p.timeout_ns : 1000000000ull;
-        while (ld_acquire(&q.ctl[SYM_DONE]) < (unsigned)q.nitems)
-            if (globaltimer_ns() - t0 > limit) {
-                ok = 0;
-                break;
-            }
-        if (!ok) atomicOr(p.err, 1);
-        s_next[0] = ok ? (int)atomicAdd(&q.ctl[SYM_FINISH], 1u) : (1 << 26) - 1;
-    }
-    __syncthreads();
-    __threadfence();
-    int unit = s_next[0];
-    for (int turn = 1; unit * 32 < p.n; turn ^= 1) {
-        if (tid == 0) s_next[turn] = (int)atomicAdd(&q.ctl[SYM_FINISH], 1u);
-        sym_finish<PK, POS == POS_SINGLE ? STAGE_F32I : STAGE_F32IX2>(
-            p, q, unit * 32, reinterpret_cast<double *>(smem_raw) + turn * 384);
-        unit = s_next[turn];
-    }
-    if (tid == 0 && atomicAdd(&q.ctl[SYM_LEFT], 1u) == gridDim.x - 1)
-        for (int k = 0; k < SYM_CTL; ++k) q.ctl[k] = 0u;
+    sym_collect<WI, POS == POS_SINGLE ? STAGE_F32I : STAGE_F32IX2>(
+        p, q, done, reinterpret_cast<double *>(smem_raw), s_next);
 }
 
 }  // namespace ppk
