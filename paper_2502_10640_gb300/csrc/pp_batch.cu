@@ -359,74 +359,33 @@ pp_status decide_slot_staging(pp_batch *b, Slot &s, int *staging)
     return PP_OK;
 }
 
-// Potential energy of one bunch: phi'_i = sum_{j != i} 1/|r'_ij| by the FP32 pair
-// kernel on freshly staged positions (scratch allocated for the call), then
-// PE = 1/2 k e^2 w^2 / L0 * sum_i phi'_i.
+// Potential energy of one bunch on freshly staged positions (scratch allocated
+// for the call): PE = k e^2 w^2 / L0 * sum over pairs of 1 / sqrt(s).
 pp_status slot_potential(pp_batch *b, Slot &s, double *pe)
 {
-    int count = 0;
-    const Variant *vs = variants(&count);
-    const Variant *v = nullptr;
-    for (int i = 0; i < count; ++i)
-        if (std::strcmp(vs[i].name, "phi32.fold64.t256r2k256") == 0) v = &vs[i];
-    if (!v) return bfail(PP_ERR_STATE, "potential kernel missing");
-    const int n = (int)s.n, npad = s.L.npad, BI = v->T * v->R;
-    const int nib = (n + BI - 1) / BI, tiles = npad / v->tile;
-    int S = std::min(tiles, std::max(1, (4 * b->sms + nib - 1) / nib));
-    const int chunk_tiles = (tiles + S - 1) / S;
-    S = (tiles + chunk_tiles - 1) / chunk_tiles;
+    const int n = (int)s.n, npad = s.L.npad;
     float4 *stage = nullptr;
-    double *phi = nullptr, *partial = nullptr;
-    unsigned *tickets = nullptr;
-    auto cleanup = [&]() {
-        cudaFree(stage);
-        cudaFree(phi);
-        cudaFree(partial);
-        cudaFree(tickets);
-    };
+    double *parts = nullptr;
     if (cudaMalloc(&stage, (size_t)npad * sizeof(float4)) != cudaSuccess ||
-        cudaMalloc(&phi, (size_t)npad * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&partial, (size_t)S * nib * BI * sizeof(double)) != cudaSuccess ||
-        cudaMalloc(&tickets, (size_t)nib * sizeof(unsigned)) != cudaSuccess) {
+        cudaMalloc(&parts, (size_t)npad * sizeof(double)) != cudaSuccess) {
         cudaGetLastError();
-        cleanup();
+        cudaFree(stage);
         return bfail(PP_ERR_NOMEM, "cannot allocate the potential-energy scratch");
     }
-    ForceArgs a{};
-    a.src = stage;
-    a.n = n;
-    a.npad = npad;
-    a.nib = nib;
-    a.nsplit = S;
-    a.jchunk = chunk_tiles * v->tile;
-    a.mode = MODE_PHI;
     const double epsl = s.eps / s.l0;
-    a.eps2d = epsl * epsl;
-    a.eps2f = (float)a.eps2d;
-    a.partial = partial;
-    a.tickets = tickets;
-    a.nipad = nib * BI;
-    a.out = phi;
-    a.err = b->d_err;
-    a.timeout_ns = b->timeout_ns;
-    double m[kMomSlots];
-    int flags[2] = {0, 0};
-    cudaError_t e = cudaMemsetAsync(tickets, 0, (size_t)nib * sizeof(unsigned), b->stream);
+    double sum = 0.0;
+    cudaError_t e = launch_stage(s.r[0], s.r[1], s.r[2], n, npad, stage, STAGE_F32, s.cx, s.cy, s.cz,
+                                 1.0 / s.l0, b->stream);
     if (e == cudaSuccess)
-        e = launch_stage(s.r[0], s.r[1], s.r[2], n, npad, stage, STAGE_F32, s.cx, s.cy, s.cz,
-                         1.0 / s.l0, b->stream);
-    if (e == cudaSuccess) e = launch_variant(*v, a, nib * S, b->stream);
+        e = launch_potential(stage, n, npad, (float)(epsl * epsl), nullptr, parts, b->mom_out,
+                             b->stream);
     if (e == cudaSuccess)
-        e = launch_moments(2, n, phi, nullptr, nullptr, nullptr, nullptr, nullptr, 0, 0, 0,
-                           b->mom_partials, b->mom_out, b->stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(m, b->mom_out, sizeof(m), cudaMemcpyDeviceToHost, b->stream);
+        e = cudaMemcpyAsync(&sum, b->mom_out, sizeof(sum), cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    cleanup();
+    cudaFree(stage);
+    cudaFree(parts);
     if (e != cudaSuccess) return bcuda(e, "potential-energy pass");
-    if (pp_status st = read_errors(b, flags)) return st;
-    if (flags[0]) return bfail(PP_ERR_TIMEOUT, "a device-side wait ran out of time");
-    *pe = 0.5 * kCoulomb * kE * kE * s.w * s.w / s.l0 * m[0];
+    *pe = kCoulomb * kE * kE * s.w * s.w / s.l0 * sum;
     return PP_OK;
 }
 

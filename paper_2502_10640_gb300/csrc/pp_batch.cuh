@@ -221,8 +221,8 @@ __device__ __forceinline__ bool batch_item(const BunchDesc *__restrict__ descs, 
     }
     bool finish = true;
     if (pe.nsplit > 1) {
-        finish = split_publish<T, R>(pe, ib, split, ax64, ay64, az64, 3, cta.s_flag);
-        if (finish) split_gather<T, R>(pe, ib, ax64, ay64, az64, 3);
+        finish = split_publish<T, R>(pe, ib, split, ax64, ay64, az64, cta.s_flag);
+        if (finish) split_gather<T, R>(pe, ib, ax64, ay64, az64);
     }
     if (finish) {
 #pragma unroll

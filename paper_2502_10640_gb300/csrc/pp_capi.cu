@@ -61,7 +61,7 @@ struct pp_ctx {
     void *stage[2] = {};           // float4 (or double4 for FP64 pair math) [npad]
     size_t stage_bytes = 0;        // per buffer: 32 bytes per entry fits every layout
     double *aos = nullptr;         // [n][3] scratch for host transfers / outputs
-    double *phi = nullptr;         // [n]
+    double *phi = nullptr;         // partial sums of the potential [npad]
     double *wts = nullptr;         // per-particle weights [npad] (null: all equal to w)
     float *wrel = nullptr;         // w_i / w as staged [npad]
     double *partial = nullptr;     // split partials
@@ -282,8 +282,6 @@ int stage_kind(const pp_ctx *c) { return force_variant(c)->stage; }
 // Pick the variant for a kind of pass.
 const Variant *pick_variant(const pp_ctx *c, int kind)
 {
-    if (kind == KIND_PHI32)
-        return variant_by_name(c->n >= 32768 ? "phi32.fold64.t256r2k256" : "phi32.fold64.t128r1k128");
     return force_variant(c);
 }
 
@@ -487,10 +485,9 @@ pp_status ensure_workspace(pp_ctx *c, const Plan &pl)
             drop_graphs(c);
         }
     }
-    const int ncomp = (pl.v->kind == KIND_PHI32) ? 1 : 3;
     if (pl.v->sym) return PP_OK;
     const size_t need = (pl.nsplit > 1 && pl.v->cluster == 0)
-                            ? (size_t)pl.nsplit * ncomp * pl.nipad * sizeof(double)
+                            ? (size_t)pl.nsplit * 3 * pl.nipad * sizeof(double)
                             : 0;
     if (need > c->partial_bytes) {
         if (c->partial) cudaFree(c->partial);
@@ -620,7 +617,7 @@ pp_status plan_pass(pp_ctx *c, int kind, bool one_sided, Plan *pl)
 // One force pass over staged sources src.
 pp_status force_pass(pp_ctx *c, int mode, const void *src, void *dst, double *out)
 {
-    const int kind = (mode == MODE_PHI) ? KIND_PHI32 : (f64_pairs(c) ? KIND_FORCE64 : KIND_FORCE32);
+    const int kind = f64_pairs(c) ? KIND_FORCE64 : KIND_FORCE32;
     // the symmetric kernels make no tile copies: the test hook takes a one-sided one
     Plan pl{};
     pp_status st = plan_pass(c, kind, c->skip_copy != 0, &pl);
@@ -782,9 +779,9 @@ pp_status take_bad_input_flag(pp_ctx *c, bool *bad)
     return PP_OK;
 }
 
-pp_status moments(pp_ctx *c, int pass, const double *x, double out[kMomSlots])
+pp_status moments(pp_ctx *c, int pass, double out[kMomSlots])
 {
-    PP_CUDA(launch_moments(pass, (int)c->n, pass == 2 ? x : c->r[0], c->r[1], c->r[2], c->v[0],
+    PP_CUDA(launch_moments(pass, (int)c->n, c->r[0], c->r[1], c->r[2], c->v[0],
                            c->v[1], c->v[2], c->cx, c->cy, c->cz, c->mom_partials, c->mom_out,
                            c->stream, c->wts));
     PP_CUDA(cudaMemcpyAsync(c->mom_host, c->mom_out, kMomSlots * sizeof(double),
@@ -800,14 +797,14 @@ pp_status choose_frame(pp_ctx *c)
 {
     double m[kMomSlots];
     c->cx = c->cy = c->cz = 0.0;
-    pp_status st = moments(c, 0, nullptr, m);
+    pp_status st = moments(c, 0, m);
     if (st != PP_OK) return st;
     const double n = (double)c->n;
     const double cx = m[0] / n, cy = m[1] / n, cz = m[2] / n;
     c->cx = cx;
     c->cy = cy;
     c->cz = cz;
-    st = moments(c, 1, nullptr, m);
+    st = moments(c, 1, m);
     if (st != PP_OK) return st;
     const double rms = std::sqrt(m[0] / n);
     double l0 = 1.0;
@@ -1697,13 +1694,13 @@ pp_status pp_diagnostics(pp_ctx *c, pp_diag *d, int with_pe)
     double m0[kMomSlots], m1[kMomSlots];
     const double scx = c->cx, scy = c->cy, scz = c->cz;
     c->cx = c->cy = c->cz = 0.0;
-    pp_status st = moments(c, 0, nullptr, m0);
+    pp_status st = moments(c, 0, m0);
     if (st != PP_OK) return st;
     const double cx = m0[0] / n, cy = m0[1] / n, cz = m0[2] / n;
     c->cx = cx;
     c->cy = cy;
     c->cz = cz;
-    st = moments(c, 1, nullptr, m1);
+    st = moments(c, 1, m1);
     c->cx = scx;
     c->cy = scy;
     c->cz = scz;
@@ -1729,19 +1726,20 @@ pp_status pp_diagnostics(pp_ctx *c, pp_diag *d, int with_pe)
     d->cz = cz;
     d->pe = NAN;
     if (with_pe) {
-        // phi'_i = sum_{j != i} 1/sqrt(|d'|^2 + eps'^2); PE = 1/2 k e^2 w^2 / L0 * sum_i phi'_i
-        // the potential pass always uses FP32 sources, staged into the idle buffer
+        // PE = k e^2 / L0 * sum over pairs of w_i w_j / sqrt(|d'|^2 + eps'^2), always on
+        // FP32 sources, staged into the idle buffer
         void *scratch = c->stage[c->parity ^ 1];
+        const double epsl = c->eps / c->l0;
         st = stage_current(c, scratch, STAGE_F32);
-        if (st == PP_OK) st = force_pass(c, MODE_PHI, scratch, nullptr, c->phi);
         if (st != PP_OK) return st;
-        st = check_device_errors(c, false);
+        PP_CUDA(launch_potential(scratch, (int)c->n, c->npad, (float)(epsl * epsl), c->wts, c->phi,
+                                 c->mom_out, c->stream));
+        PP_CUDA(cudaMemcpyAsync(c->mom_host, c->mom_out, sizeof(double), cudaMemcpyDeviceToHost,
+                                c->stream));
+        st = check_device_errors(c, false);   // synchronises
         if (st != PP_OK) return st;
-        double mp[kMomSlots];
-        st = moments(c, 2, c->phi, mp);
-        if (st != PP_OK) return st;
-        // sum_i w_i phi'_i (weights) or sum_i phi'_i (equal weights, times w)
-        d->pe = 0.5 * kCoulomb * kE * kE * c->w / c->l0 * mp[0] * (c->wts ? 1.0 : c->w);
+        // sum_i w_i phi_i (weights) or sum_i phi_i (equal weights, times w)
+        d->pe = kCoulomb * kE * kE * c->w / c->l0 * c->mom_host[0] * (c->wts ? 1.0 : c->w);
     }
     return PP_OK;
 }

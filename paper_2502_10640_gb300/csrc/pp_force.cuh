@@ -33,8 +33,7 @@ namespace ppk {
 enum Mode : int {
     MODE_STEP = 0,    // a_{n+1} from staged r_{n+1}; epilogue: Eq. G recompute, Eq. H, stage r_{n+2}
     MODE_FIELDS = 1,  // E = escale * sum, written [N][3]; state untouched
-    MODE_INIT = 2,    // a_0 from staged r_0; epilogue: store a_0, stage r_1 (Eq. G)
-    MODE_PHI = 3      // phi'_i = sum_{j != i} 1/sqrt(s); written [N]
+    MODE_INIT = 2     // a_0 from staged r_0; epilogue: store a_0, stage r_1 (Eq. G)
 };
 
 enum Acc : int { ACC_FP64FOLD = 0, ACC_KAHAN = 1, ACC_FP64FULL = 2 };
@@ -59,7 +58,7 @@ struct ForceArgs {
     double *v[3];
     double *a[3];
     void *dst;              // staging written by the epilogue (float4 or double4)
-    double *out;            // fields [n][3] (MODE_FIELDS) or phi [n] (MODE_PHI)
+    double *out;            // fields [n][3] (MODE_FIELDS)
     const float *wrel;      // per-particle weight / reference weight, or null (all 1)
     double cscale;          // a = cscale * sum
     double escale;          // E = escale * sum
@@ -177,10 +176,6 @@ __device__ __forceinline__ void finish_particle(const ForceArgs &p, int i, doubl
         p.out[3 * (size_t)i + 0] = p.escale * sx;
         p.out[3 * (size_t)i + 1] = p.escale * sy;
         p.out[3 * (size_t)i + 2] = p.escale * sz;
-        return;
-    }
-    if (p.mode == MODE_PHI) {
-        p.out[i] = sx;
         return;
     }
     const double an[3] = {p.cscale * sx, p.cscale * sy, p.cscale * sz};
@@ -422,19 +417,17 @@ __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
 template <int T, int R>
 __device__ __forceinline__ bool split_publish(const ForceArgs &p, int ib, int split,
                                               const double (&sx)[R], const double (&sy)[R],
-                                              const double (&sz)[R], int ncomp, int *s_flag)
+                                              const double (&sz)[R], int *s_flag)
 {
     const int tid = threadIdx.x;
     const size_t stride = (size_t)p.nipad;
-    double *base = p.partial + (size_t)split * ncomp * stride;
+    double *base = p.partial + (size_t)split * 3 * stride;
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int i = ib * T * R + r * T + tid;
         base[i] = sx[r];
-        if (ncomp == 3) {
-            base[stride + i] = sy[r];
-            base[2 * stride + i] = sz[r];
-        }
+        base[stride + i] = sy[r];
+        base[2 * stride + i] = sz[r];
     }
     __threadfence();
     __syncthreads();
@@ -455,7 +448,7 @@ __device__ __forceinline__ bool split_publish(const ForceArgs &p, int ib, int sp
 // is a fixed function of S, so results stay bitwise reproducible.
 template <int T, int R>
 __device__ __forceinline__ void split_gather(const ForceArgs &p, int ib, double (&sx)[R],
-                                             double (&sy)[R], double (&sz)[R], int ncomp)
+                                             double (&sy)[R], double (&sz)[R])
 {
     constexpr int U = 4;
     const int tid = threadIdx.x;
@@ -473,10 +466,10 @@ __device__ __forceinline__ void split_gather(const ForceArgs &p, int ib, double 
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const int s = s0 + u;
-                const double *base = p.partial + (size_t)s * ncomp * stride + i;
+                const double *base = p.partial + (size_t)s * 3 * stride + i;
 #pragma unroll
                 for (int c = 0; c < 3; ++c)
-                    v[c][u] = (s < p.nsplit && c < ncomp) ? ld_cg(base + c * stride) : 0.0;
+                    v[c][u] = s < p.nsplit ? ld_cg(base + c * stride) : 0.0;
             }
 #pragma unroll
             for (int c = 0; c < 3; ++c)
@@ -601,96 +594,13 @@ __global__ void __launch_bounds__(T, MINB) force_f32_kernel(const ForceArgs p)
         }
     }
     if (p.nsplit > 1) {
-        if (!split_publish<T, R>(p, ib, split, dx64, dy64, dz64, 3, &s_flag)) return;
-        split_gather<T, R>(p, ib, dx64, dy64, dz64, 3);
+        if (!split_publish<T, R>(p, ib, split, dx64, dy64, dz64, &s_flag)) return;
+        split_gather<T, R>(p, ib, dx64, dy64, dz64);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
         finish_particle<SPLIT ? STAGE_F32X2 : STAGE_F32>(p, i0 + r * T + tid, dx64[r], dy64[r],
                                                          dz64[r]);
-}
-
-// ---- potential: phi'_i = sum_{j != i, s > 0} 1/sqrt(s), FP32 pairs, FP64 fold ----
-template <int T, int R, int TILE, int STAGES>
-__global__ void __launch_bounds__(T) phi_f32_kernel(const ForceArgs p)
-{
-    constexpr int BI = T * R;
-    extern __shared__ __align__(128) unsigned char smem_raw[];
-    __shared__ uint64_t bar_full[STAGES], bar_empty[STAGES];
-    __shared__ int s_abort, s_flag;
-
-    const int tid = threadIdx.x;
-    const int ib = blockIdx.x % p.nib;
-    const int split = blockIdx.x / p.nib;
-    const int i0 = ib * BI;
-    const int j0 = split * p.jchunk;
-    const int j1 = min(j0 + p.jchunk, p.npad);
-    const int ntiles = (j1 - j0) / TILE;
-
-    Ring<float4, TILE, STAGES> rg{reinterpret_cast<float4 *>(smem_raw), nullptr, bar_full, bar_empty};
-    if (tid == 0) {
-        for (int s = 0; s < STAGES; ++s) {
-            mbar_init(&bar_full[s], 1);
-            mbar_init(&bar_empty[s], T / 32);
-        }
-        s_abort = 0;
-        fence_barrier_init();
-    }
-    __syncthreads();
-
-    const float4 *src = static_cast<const float4 *>(p.src);
-    float xi[R], yi[R], zi[R];
-    int gi[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const int i = i0 + r * T + tid;
-        gi[r] = i;
-        const float4 q = (i < p.n) ? src[i] : make_float4(-1e18f, -1e18f, -1e18f, 0.f);
-        xi[r] = q.x;
-        yi[r] = q.y;
-        zi[r] = q.z;
-    }
-    double acc[R], dummy[R];
-#pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = dummy[r] = 0.0;
-    const float eps2 = p.eps2f;
-    int issued = 0, seen = 0;
-    const bool ok = run_tiles<float4, T, TILE, STAGES, false>(
-        p, rg, j0, ntiles, issued, seen, [&](const float4 *tile, const float4 *, int jfirst) {
-            float f[R];
-#pragma unroll
-            for (int r = 0; r < R; ++r) f[r] = 0.f;
-            for (int j = 0; j < TILE; ++j) {
-                const float4 q = tile[j];
-#pragma unroll
-                for (int r = 0; r < R; ++r) {
-                    const float dx = xi[r] - q.x;
-                    const float dy = yi[r] - q.y;
-                    const float dz = zi[r] - q.z;
-                    const float s = fmaf(dz, dz, fmaf(dy, dy, fmaf(dx, dx, eps2)));
-                    // padding sources carry q.w = 0
-                    const float term = (s > 0.f && jfirst + j != gi[r]) ? q.w * rsqrt_sfu(s) : 0.f;
-                    f[r] += term;
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < R; ++r) acc[r] += (double)f[r];
-        });
-    if (!ok) {
-        s_abort = 1;
-        atomicOr(p.err, 1);
-    }
-    __syncthreads();
-    if (s_abort) {
-        ring_drain(p, rg, issued, seen, ntiles);
-        return;
-    }
-    if (p.nsplit > 1) {
-        if (!split_publish<T, R>(p, ib, split, acc, dummy, dummy, 1, &s_flag)) return;
-        split_gather<T, R>(p, ib, acc, dummy, dummy, 1);
-    }
-#pragma unroll
-    for (int r = 0; r < R; ++r) finish_particle<STAGE_F32>(p, i0 + r * T + tid, acc[r], 0.0, 0.0);
 }
 
 // ---- FP64 pair math and accumulation (comparison path) ---------------------
@@ -765,8 +675,8 @@ __global__ void __launch_bounds__(T) force_f64_kernel(const ForceArgs p)
         return;
     }
     if (p.nsplit > 1) {
-        if (!split_publish<T, R>(p, ib, split, ax, ay, az, 3, &s_flag)) return;
-        split_gather<T, R>(p, ib, ax, ay, az, 3);
+        if (!split_publish<T, R>(p, ib, split, ax, ay, az, &s_flag)) return;
+        split_gather<T, R>(p, ib, ax, ay, az);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
@@ -1156,7 +1066,7 @@ __device__ __forceinline__ void guard_thresholds(const f2_t (&X)[R], const f2_t 
 template <int T, int R, int TILE, int STAGES, int MINB, bool SMEM_ACC = false,
           bool WEIGHTED = false, bool SPLITPOS = false, int UNROLL = 2, bool KAHAN = false,
           int GUARD = 0>
-__global__ void __launch_bounds__(T, MINB) force_f32x2_kernel(const ForceArgs p)
+__device__ __forceinline__ void force_f32x2_body(const ForceArgs &p)
 {
     static_assert(!(GUARD != 0 && SPLITPOS), "guarded staging sums the hi parts only");
     // the ring carries the lo parts too with hi/lo staging and with the box guard
@@ -1327,13 +1237,22 @@ __global__ void __launch_bounds__(T, MINB) force_f32x2_kernel(const ForceArgs p)
         }
     }
     if (p.nsplit > 1) {
-        if (!split_publish<T, R>(p, ib, split, ax64, ay64, az64, 3, &s_flag)) return;
-        split_gather<T, R>(p, ib, ax64, ay64, az64, 3);
+        if (!split_publish<T, R>(p, ib, split, ax64, ay64, az64, &s_flag)) return;
+        split_gather<T, R>(p, ib, ax64, ay64, az64);
     }
 #pragma unroll
     for (int r = 0; r < R; ++r)
         finish_particle<(SPLITPOS || GUARD != 0) ? STAGE_F32IX2 : STAGE_F32I>(p, i0 + r * T + tid,
                                                                          ax64[r], ay64[r], az64[r]);
+}
+
+template <int T, int R, int TILE, int STAGES, int MINB, bool SMEM_ACC = false,
+          bool WEIGHTED = false, bool SPLITPOS = false, int UNROLL = 2, bool KAHAN = false,
+          int GUARD = 0>
+__global__ void __launch_bounds__(T, MINB) force_f32x2_kernel(const ForceArgs p)
+{
+    force_f32x2_body<T, R, TILE, STAGES, MINB, SMEM_ACC, WEIGHTED, SPLITPOS, UNROLL, KAHAN, GUARD>(
+        p);
 }
 
 

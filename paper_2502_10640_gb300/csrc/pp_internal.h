@@ -37,7 +37,7 @@ constexpr double kCoulomb = 1.0 / (4.0 * kPi * kEps0);  // 1/(4 pi eps0), Eq. A
 // Staged arrays are padded to a multiple of this many entries.
 constexpr int kPad = 1024;
 
-enum Kind : int { KIND_FORCE32 = 0, KIND_PHI32 = 1, KIND_FORCE64 = 2, KIND_FORCE32W = 3 };
+enum Kind : int { KIND_FORCE32 = 0, KIND_FORCE64 = 2, KIND_FORCE32W = 3 };
 
 struct Variant {
     const char *name;
@@ -174,7 +174,6 @@ cudaError_t launch_export_state(double *const r[3], double *const v[3], double *
 //  pass 0: sums of x, y, z                                     -> out[0..2]
 //  pass 1: sum |r-c|^2, sum w|v|^2, sum w vx, w vy, w vz, sum x^2,
 //          sum vx^2, sum x vx (out[0..7]); max x, max vx (out[10], out[11])
-//  pass 2: sum of w times the values in x (one array)          -> out[0]
 // wts: per-particle weights, or null for weight 1.
 constexpr int kMomSlots = 12;
 constexpr int kMomBlocks = 240;
@@ -182,6 +181,13 @@ cudaError_t launch_moments(int pass, int n, const double *x, const double *y, co
                            const double *vx, const double *vy, const double *vz, double cx,
                            double cy, double cz, double *block_partials, double *out,
                            cudaStream_t s, const double *wts = nullptr);
+
+// sum over unordered pairs of w_i w_j / sqrt(s) over the staged sources src
+// (STAGE_F32, npad entries, their weight slot w_j), zero-distance pairs left
+// out: out[0].  wts: per-particle weights w_i, or null for 1.  partials: room for
+// npad doubles (pp_potential.cu).
+cudaError_t launch_potential(const void *src, int n, int npad, float eps2, const double *wts,
+                             double *partials, double *out, cudaStream_t s);
 
 // Sums of |a - b|^2 and |b|^2 over n3 doubles: partials[2k], partials[2k+1] for
 // k < kDiffBlocks (a fixed reduction order; the host adds the blocks in order).

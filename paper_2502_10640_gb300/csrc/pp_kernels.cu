@@ -65,14 +65,6 @@ Variant make_cluster(const char *name)
 }
 
 template <int T, int R, int TILE, int STAGES>
-Variant make_phi(const char *name)
-{
-    return Variant{name, KIND_PHI32, ACC_FP64FOLD, STAGE_F32, T, R, TILE, STAGES,
-                   reinterpret_cast<const void *>(&phi_f32_kernel<T, R, TILE, STAGES>),
-                   (size_t)STAGES * TILE * sizeof(float4), 0, POS_SINGLE};
-}
-
-template <int T, int R, int TILE, int STAGES>
 Variant make_f64(const char *name)
 {
     return Variant{name, KIND_FORCE64, ACC_FP64FULL, STAGE_F64, T, R, TILE, STAGES,
@@ -148,9 +140,7 @@ const Variant kVariants[] = {
     make_f32x2<128, 4, 512, 3, 4, true, true>("f32x2w.sfold64.t128r4k512m4"),
     make_f32x2<128, 2, 128, 4, 4, false, true>("f32x2w.fold64.t128r2k128"),
     make_f32x2<64, 1, 128, 4, 8, false, true>("f32x2w.fold64.t64r1k128"),
-    // potential (diagnostics) and all-FP64 comparison path
-    make_phi<256, 2, 256, 4>("phi32.fold64.t256r2k256"),
-    make_phi<128, 1, 128, 4>("phi32.fold64.t128r1k128"),
+    // all-FP64 comparison path
     make_f64<128, 2, 128, 3>("f64.full.t128r2k128"),
 };
 

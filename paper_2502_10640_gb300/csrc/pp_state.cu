@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(kMomThreads)
             acc[0] += x[i];
             acc[1] += y[i];
             acc[2] += z[i];
-        } else if (pass == 1) {
+        } else {
             const double dx = x[i] - cx, dy = y[i] - cy, dz = z[i] - cz;
             const double wi = wts ? wts[i] : 1.0;
             acc[0] += dx * dx + dy * dy + dz * dz;
@@ -192,8 +192,6 @@ __global__ void __launch_bounds__(kMomThreads)
             acc[7] += x[i] * vx[i];
             acc[10] = fmax(acc[10], x[i]);
             acc[11] = fmax(acc[11], vx[i]);
-        } else {
-            acc[0] += wts ? wts[i] * x[i] : x[i];
         }
     }
     for (int k = 0; k < kMomSlots; ++k) block_sum(sh, k, acc[k]);
@@ -212,17 +210,22 @@ __global__ void __launch_bounds__(kMomThreads)
         partials[blockIdx.x * kMomSlots + threadIdx.x] = sh[threadIdx.x * kMomThreads];
 }
 
-__global__ void moments_finish_kernel(const double *__restrict__ partials, int nblocks,
-                                      double *out)
+// One warp per slot: lane l adds blocks l, l + 32, ..., then a fixed tree (a single
+// thread per slot took 20 us over 240 blocks).
+__global__ void __launch_bounds__(32 * kMomSlots)
+    moments_finish_kernel(const double *__restrict__ partials, int nblocks, double *out)
 {
-    const int k = threadIdx.x;
-    if (k >= kMomSlots) return;
+    const int k = threadIdx.x >> 5, lane = threadIdx.x & 31;
     double acc = (k >= 10) ? -INFINITY : 0.0;
-    for (int b = 0; b < nblocks; ++b) {
+    for (int b = lane; b < nblocks; b += 32) {
         const double v = partials[b * kMomSlots + k];
         acc = (k >= 10) ? fmax(acc, v) : acc + v;
     }
-    out[k] = acc;
+    for (int h = 16; h > 0; h >>= 1) {
+        const double v = __shfl_down_sync(0xffffffffu, acc, h);
+        acc = (k >= 10) ? fmax(acc, v) : acc + v;
+    }
+    if (lane == 0) out[k] = acc;
 }
 
 int grid_for(int n, int threads)
@@ -334,11 +337,13 @@ cudaError_t launch_moments(int pass, int n, const double *x, const double *y, co
                            double cy, double cz, double *block_partials, double *out,
                            cudaStream_t s, const double *wts)
 {
-    moments_kernel<<<kMomBlocks, kMomThreads, 0, s>>>(pass, n, x, y, z, vx, vy, vz, cx, cy, cz,
-                                                      block_partials, wts);
+    const int full = (n + kMomThreads - 1) / kMomThreads;
+    const int blocks = full < kMomBlocks ? full : kMomBlocks;
+    moments_kernel<<<blocks, kMomThreads, 0, s>>>(pass, n, x, y, z, vx, vy, vz, cx, cy, cz,
+                                                  block_partials, wts);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    moments_finish_kernel<<<1, 32, 0, s>>>(block_partials, kMomBlocks, out);
+    moments_finish_kernel<<<1, 32 * kMomSlots, 0, s>>>(block_partials, blocks, out);
     return cudaGetLastError();
 }
 
