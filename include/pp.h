@@ -302,7 +302,7 @@ pp_status pp_check_mapped(const void *p, int64_t bytes);
  * runs inside a memory arena owned by a host framework, code that must not
  * trigger the allocator's implicit synchronisation, plug-ins restricted to the
  * buffers they are handed).  Every intermediate lives in one fixed device
- * array of 4.09 MB that each GPU loading this library holds until the
+ * array of 3.67 MB that each GPU loading this library holds until the
  * process exits; N above PP_FIELDS_NOALLOC_MAX_N returns PP_ERR_ARG.
  *
  * All calls on a device share that array and it keeps the last call's
@@ -311,9 +311,8 @@ pp_status pp_check_mapped(const void *p, int64_t bytes);
  * device looks up the array's device address (cudaGetSymbolAddress with that
  * device current); make that first call before any stream capture.  The
  * lookup is repeated if the device's context has been recreated since (after
- * cudaDeviceReset, for instance).  The call synchronises `stream` three times
- * before it returns: twice mid-call, to read the centroid and RMS radius that
- * fix the staging frame, and once at the end, to read the error word.
+ * cudaDeviceReset, for instance).  The call synchronises `stream` once, before it
+ * returns, to read the error words.
  * Errors: PP_ERR_ARG (size, null pointer, non-finite input), PP_ERR_TIMEOUT,
  * PP_ERR_CUDA; message via pp_last_error(NULL).
  */

@@ -11,12 +11,18 @@
 // allocations, code that must never trigger the allocator's implicit device
 // synchronisation in a latency-critical loop, or a plug-in that may only use
 // the buffers it is handed.  This entry point serves them.  It takes device
-// inputs and outputs from the caller and keeps every intermediate (SoA copy of
-// the positions, staged hi/lo float4 sources, j-split partial sums, tickets,
-// moment partials, error word) in one file-scope __device__ array of fixed size.
+// inputs and outputs from the caller and keeps every intermediate (staged hi/lo
+// sources, j-split partial sums, tickets, moment partials, frame, error words)
+// in one file-scope __device__ array of fixed size.
+//
+// The call is latency: the pair sum itself takes 2 us at N = 900.  So the
+// staging frame (centroid, RMS radius, length unit) never comes to the host:
+// each kernel finishes the reduction that the one before it left per block, the
+// force kernel reads its two scale factors from the array, and the host waits
+// once, at the end (before: ten launches and three waits, 190 us at N = 900).
 //
 // The array exists on every GPU that loads this library, for the lifetime of
-// the process (kScratchBytes, 4.09 MB).  All calls on a device share it
+// the process (kScratchBytes, 3.67 MB).  All calls on a device share it
 // and it keeps the last call's contents; the entry point clears the parts that
 // must start at zero (tickets, error word) on every call.  Calls whose work
 // overlaps on the GPU (several host threads, or several streams) race on the
@@ -45,21 +51,31 @@ namespace {
 
 constexpr int kNoAllocMaxN = PP_FIELDS_NOALLOC_MAX_N;    // largest N accepted
 constexpr int kNoAllocMaxSplit = 8;                      // j-chunks per i-block
-constexpr int kT = 128, kR = 2, kTile = 128, kStages = 4;
-constexpr int kBI = kT * kR;
+constexpr int kTile = 128, kStages = 4;
+// Targets per block: 64 (one per thread, many CTAs) up to kWideN, 256 above.
+constexpr int kWideN = 4096;
 constexpr int kMaxPad = (kNoAllocMaxN + kPad - 1) / kPad * kPad;
-constexpr int kMaxNib = (kNoAllocMaxN + kBI - 1) / kBI;
+constexpr int kMaxNib = (kNoAllocMaxN + 255) / 256;
+static_assert(kMaxNib >= (kWideN + 63) / 64, "tickets for either blocking");
+constexpr int kNaThreads = 256;
+constexpr int kMaxBlocks = (kNoAllocMaxN + kNaThreads - 1) / kNaThreads;   // of the O(N) kernels
+
+// What the force kernel needs of the staging frame.
+struct NaFrame {
+    float eps2f;
+    double escale;
+};
 
 // Byte offsets of the parts of the scratch array (each 256-byte aligned).
 constexpr size_t align256(size_t x) { return (x + 255) / 256 * 256; }
-constexpr size_t kOffSoa = 0;                                              // 3 x double[max_pad]
-constexpr size_t kOffStage = align256(kOffSoa + 3 * sizeof(double) * kMaxPad);  // float4[2 max_pad]
+constexpr size_t kOffStage = 0;                                    // hi, lo: float4[2 max_pad]
 constexpr size_t kOffPartial = align256(kOffStage + 2 * sizeof(float4) * kMaxPad);
 constexpr size_t kOffTickets =
-    align256(kOffPartial + sizeof(double) * kNoAllocMaxSplit * 3 * (size_t)kMaxNib * kBI);
-constexpr size_t kOffMomPart = align256(kOffTickets + sizeof(unsigned) * kMaxNib);
-constexpr size_t kOffMomOut = align256(kOffMomPart + sizeof(double) * kMomBlocks * kMomSlots);
-constexpr size_t kOffErr = align256(kOffMomOut + sizeof(double) * kMomSlots);
+    align256(kOffPartial + sizeof(double) * kNoAllocMaxSplit * 3 * (size_t)kMaxNib * 256);
+constexpr size_t kOffSums = align256(kOffTickets + sizeof(unsigned) * kMaxNib);  // per block: x, y, z
+constexpr size_t kOffSquares = align256(kOffSums + 3 * sizeof(double) * kMaxBlocks);
+constexpr size_t kOffFrame = align256(kOffSquares + sizeof(double) * kMaxBlocks);
+constexpr size_t kOffErr = align256(kOffFrame + sizeof(NaFrame));
 constexpr size_t kScratchBytes = align256(kOffErr + 2 * sizeof(int));
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -135,6 +151,123 @@ pp_status scratch_address(int dev, unsigned char **out)
     return PP_OK;
 }
 
+// Sum over the block's threads of up to three values, in a fixed order; the
+// result is returned on every thread.
+__device__ double3 block_sum3(double x, double y, double z)
+{
+    __shared__ double sh[3][kNaThreads / 32];
+    for (int h = 16; h > 0; h >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, h);
+        y += __shfl_xor_sync(0xffffffffu, y, h);
+        z += __shfl_xor_sync(0xffffffffu, z, h);
+    }
+    __syncthreads();   // sh may still be read from the call before
+    if ((threadIdx.x & 31) == 0) {
+        sh[0][threadIdx.x >> 5] = x;
+        sh[1][threadIdx.x >> 5] = y;
+        sh[2][threadIdx.x >> 5] = z;
+    }
+    __syncthreads();
+    x = y = z = 0.0;
+    for (int w = 0; w < kNaThreads / 32; ++w) {
+        x += sh[0][w];
+        y += sh[1][w];
+        z += sh[2][w];
+    }
+    return make_double3(x, y, z);
+}
+
+// The centroid from the per-block sums (every block adds them itself).
+__device__ double3 centroid(const double *sums, int blocks, int n)
+{
+    const int t = threadIdx.x;
+    const bool on = t < blocks;
+    const double3 s = block_sum3(on ? sums[3 * t] : 0.0, on ? sums[3 * t + 1] : 0.0,
+                                 on ? sums[3 * t + 2] : 0.0);
+    return make_double3(s.x / n, s.y / n, s.z / n);
+}
+
+// Sums of the positions per block, the check that they are finite (err[1]) and the
+// clear of the tickets.
+__global__ void __launch_bounds__(kNaThreads)
+    na_sums_kernel(const double *__restrict__ pos, int n, double *sums, unsigned *tickets,
+                   int ntickets, int *err)
+{
+    const int i = blockIdx.x * kNaThreads + threadIdx.x;
+    if (i < ntickets) tickets[i] = 0u;
+    double x = 0.0, y = 0.0, z = 0.0;
+    if (i < n) {
+        x = pos[3 * i];
+        y = pos[3 * i + 1];
+        z = pos[3 * i + 2];
+        if (!(isfinite(x) && isfinite(y) && isfinite(z))) err[1] = 1;
+    }
+    const double3 s = block_sum3(x, y, z);
+    if (threadIdx.x == 0) {
+        sums[3 * blockIdx.x] = s.x;
+        sums[3 * blockIdx.x + 1] = s.y;
+        sums[3 * blockIdx.x + 2] = s.z;
+    }
+}
+
+// Sums of the squared distances from the centroid per block.
+__global__ void __launch_bounds__(kNaThreads)
+    na_squares_kernel(const double *__restrict__ pos, int n, const double *sums, int blocks,
+                      double *squares)
+{
+    const double3 c = centroid(sums, blocks, n);
+    const int i = blockIdx.x * kNaThreads + threadIdx.x;
+    double q = 0.0;
+    if (i < n) {
+        const double dx = pos[3 * i] - c.x, dy = pos[3 * i + 1] - c.y, dz = pos[3 * i + 2] - c.z;
+        q = dx * dx + dy * dy + dz * dz;
+    }
+    const double3 s = block_sum3(q, 0.0, 0.0);
+    if (threadIdx.x == 0) squares[blockIdx.x] = s.x;
+}
+
+// The frame (centre = centroid, L0 = the power of two nearest the RMS radius) and
+// the staged hi/lo sources with their padding.
+__global__ void __launch_bounds__(kNaThreads)
+    na_stage_kernel(const double *__restrict__ pos, int n, int npad, const double *sums,
+                    const double *squares, int blocks, double eps, double field_scale, void *stage,
+                    NaFrame *frame)
+{
+    const double3 c = centroid(sums, blocks, n);
+    const int t = threadIdx.x;
+    const double q = block_sum3(t < blocks ? squares[t] : 0.0, 0.0, 0.0).x;
+    const double rms = sqrt(q / n);
+    double l0 = 1.0;
+    if (isfinite(rms) && rms > 0.0) {
+        const int e = (int)llround(log2(rms));
+        l0 = ldexp(1.0, e < -200 ? -200 : (e > 200 ? 200 : e));
+    }
+    const int i = blockIdx.x * kNaThreads + t;
+    if (i < n)
+        store_staged<STAGE_F32IX2>(stage, npad, i, pos[3 * i], pos[3 * i + 1], pos[3 * i + 2], c.x,
+                                   c.y, c.z, 1.0 / l0);
+    else if (i < npad)
+        store_padding<STAGE_F32IX2>(stage, npad, i);
+    if (i == 0) {
+        const double epsl = eps / l0;
+        frame->eps2f = (float)(epsl * epsl);
+        frame->escale = field_scale / (l0 * l0);
+    }
+}
+
+// The packed hi/lo force kernel with the frame taken from device memory; leaves
+// E_out alone if the input was not finite (bad).
+template <int T, int R>
+__global__ void __launch_bounds__(T, 512 / T)
+    na_force_kernel(const ForceArgs a, const NaFrame *frame, const int *bad)
+{
+    if (*bad) return;
+    ForceArgs p = a;
+    p.eps2f = frame->eps2f;
+    p.escale = frame->escale;
+    force_f32x2_body<T, R, kTile, kStages, 512 / T, false, false, true>(p);
+}
+
 }  // namespace
 
 extern "C" pp_status pp_fields_noalloc(int64_t N, double w, double softening, const double *pos,
@@ -154,44 +287,30 @@ extern "C" pp_status pp_fields_noalloc(int64_t N, double w, double softening, co
 
     const int n = (int)N;
     const int npad = (n + kPad - 1) / kPad * kPad;
-    double *sx = reinterpret_cast<double *>(base + kOffSoa);
-    double *sy = sx + kMaxPad, *sz = sy + kMaxPad;
-    float4 *stage = reinterpret_cast<float4 *>(base + kOffStage);
-    double *partial = reinterpret_cast<double *>(base + kOffPartial);
+    void *stage = base + kOffStage;
+    double *sums = reinterpret_cast<double *>(base + kOffSums);
+    double *squares = reinterpret_cast<double *>(base + kOffSquares);
     unsigned *tickets = reinterpret_cast<unsigned *>(base + kOffTickets);
-    double *mom_part = reinterpret_cast<double *>(base + kOffMomPart);
-    double *mom_out = reinterpret_cast<double *>(base + kOffMomOut);
+    NaFrame *frame = reinterpret_cast<NaFrame *>(base + kOffFrame);
     int *err = reinterpret_cast<int *>(base + kOffErr);
 
-    const int nib = (n + kBI - 1) / kBI;
-    NA_CUDA(cudaMemsetAsync(tickets, 0, sizeof(unsigned) * nib, st));
+    const bool wide = n > kWideN;
+    const int bi = wide ? 256 : 64;
+    const int nib = (n + bi - 1) / bi;
+    const int blocks = (n + kNaThreads - 1) / kNaThreads;
     NA_CUDA(cudaMemsetAsync(err, 0, 2 * sizeof(int), st));
-    NA_CUDA(launch_aos_to_soa(pos, n, sx, sy, sz, err + 1, st));
+    na_sums_kernel<<<blocks, kNaThreads, 0, st>>>(pos, n, sums, tickets, nib, err);
+    NA_CUDA(cudaGetLastError());
+    na_squares_kernel<<<blocks, kNaThreads, 0, st>>>(pos, n, sums, blocks, squares);
+    NA_CUDA(cudaGetLastError());
+    na_stage_kernel<<<npad / kNaThreads, kNaThreads, 0, st>>>(
+        pos, n, npad, sums, squares, blocks, softening, -kCoulomb * kE * w, stage, frame);
+    NA_CUDA(cudaGetLastError());
 
-    // staging frame: centroid and the power of two nearest the RMS radius
-    double m[kMomSlots];
-    NA_CUDA(launch_moments(0, n, sx, sy, sz, sx, sy, sz, 0, 0, 0, mom_part, mom_out, st));
-    NA_CUDA(cudaMemcpyAsync(m, mom_out, sizeof(m), cudaMemcpyDeviceToHost, st));
-    NA_CUDA(cudaStreamSynchronize(st));
-    const double cx = m[0] / n, cy = m[1] / n, cz = m[2] / n;
-    NA_CUDA(launch_moments(1, n, sx, sy, sz, sx, sy, sz, cx, cy, cz, mom_part, mom_out, st));
-    NA_CUDA(cudaMemcpyAsync(m, mom_out, sizeof(m), cudaMemcpyDeviceToHost, st));
-    int flags[2] = {0, 0};
-    NA_CUDA(cudaMemcpyAsync(flags, err, sizeof(flags), cudaMemcpyDeviceToHost, st));
-    NA_CUDA(cudaStreamSynchronize(st));
-    if (flags[1]) return na_fail(PP_ERR_ARG, "non-finite position");
-    const double rms = std::sqrt(m[0] / n);
-    double l0 = 1.0;
-    if (std::isfinite(rms) && rms > 0.0) {
-        int e = (int)std::lround(std::log2(rms));
-        e = e < -200 ? -200 : (e > 200 ? 200 : e);
-        l0 = std::ldexp(1.0, e);
-    }
-    // hi parts at stage[0, npad), lo parts at stage[npad, 2 npad)
-    NA_CUDA(launch_stage(sx, sy, sz, n, npad, stage, STAGE_F32X2, cx, cy, cz, 1.0 / l0, st));
-
+    // a tile per CTA while the partial sums fit (64-target blocks), at most 8 chunks above
     const int tiles = npad / kTile;
-    const int nsplit_req = tiles < kNoAllocMaxSplit ? tiles : kNoAllocMaxSplit;
+    const int most = wide ? kNoAllocMaxSplit : kNoAllocMaxSplit * kMaxNib * 256 / (nib * bi);
+    const int nsplit_req = tiles < most ? tiles : most;
     const int chunk_tiles = (tiles + nsplit_req - 1) / nsplit_req;
     ForceArgs a{};
     a.src = stage;
@@ -201,27 +320,22 @@ extern "C" pp_status pp_fields_noalloc(int64_t N, double w, double softening, co
     a.jchunk = chunk_tiles * kTile;
     a.nsplit = (tiles + chunk_tiles - 1) / chunk_tiles;
     a.mode = MODE_FIELDS;
-    const double epsl = softening / l0;
-    a.eps2d = epsl * epsl;
-    a.eps2f = (float)a.eps2d;
-    a.partial = partial;
+    a.partial = reinterpret_cast<double *>(base + kOffPartial);
     a.tickets = tickets;
-    a.nipad = nib * kBI;
+    a.nipad = nib * bi;
     a.out = E_out;
-    a.escale = -kCoulomb * kE * w / (l0 * l0);
-    a.cx = cx;
-    a.cy = cy;
-    a.cz = cz;
-    a.inv_l0 = 1.0 / l0;
     a.err = err;
     a.timeout_ns = 1000000000ull;
-    void *args[] = {&a};
-    const void *fn = reinterpret_cast<const void *>(
-        &force_f32_kernel<kT, kR, kTile, kStages, ACC_FP64FOLD, 4, true>);
-    NA_CUDA(cudaLaunchKernel(fn, dim3(nib * a.nsplit), dim3(kT), args,
-                             (size_t)kStages * kTile * sizeof(float4) * 2, st));
+    const size_t smem = (size_t)kStages * kTile * sizeof(float4) * 2;
+    if (wide)
+        na_force_kernel<128, 2><<<nib * a.nsplit, 128, smem, st>>>(a, frame, err + 1);
+    else
+        na_force_kernel<64, 1><<<nib * a.nsplit, 64, smem, st>>>(a, frame, err + 1);
+    NA_CUDA(cudaGetLastError());
+    int flags[2] = {0, 0};
     NA_CUDA(cudaMemcpyAsync(flags, err, sizeof(flags), cudaMemcpyDeviceToHost, st));
     NA_CUDA(cudaStreamSynchronize(st));
+    if (flags[1]) return na_fail(PP_ERR_ARG, "non-finite position");
     if (flags[0]) return na_fail(PP_ERR_TIMEOUT, "a device-side wait ran out of time");
     return PP_OK;
 }
