@@ -867,6 +867,10 @@ constexpr int64_t kResidentAutoMaxN = kResidentMaxN;
 // CTA size: 512 threads from this N on (more warps to hide latency once the
 // pair work dominates), 256 below (fewer partial sums per target).
 constexpr int64_t kResidentWideN = 3072;
+// Two targets per thread from this N on (us per step with one and two: 13.1 / 12.9 at N =
+// 5000, 18.0 / 17.3 at 6144, 29.7 / 28.2 at 8192, 44.6 / 39.6 at 10000, 62.3 / 58.1 at
+// 12288, hi/lo 26.2 / 24.9 at 6144; below, 5.05 / 5.12 at 2048).
+constexpr int64_t kResidentPairN = 5000;
 // Steps per cooperative launch (bounds a launch to tens of milliseconds).
 constexpr int64_t kResidentMaxSteps = 4096;
 // Largest grid of the resident kernel (one CTA per SM).
@@ -874,7 +878,7 @@ constexpr int kResidentMaxGrid = 256;
 
 struct ResidentPlan {
     bool ok = false;
-    int form = 0, grid = 0, threads = 0, bt = 0, q = 0, chunk = 0, nsrc = 0;
+    int form = 0, grid = 0, threads = 0, targets = 0, bt = 0, q = 0, chunk = 0, nsrc = 0;
 };
 
 // Can pp_step use the resident kernel, and how is the work split?
@@ -909,11 +913,13 @@ ResidentPlan compute_resident_plan(const pp_ctx *c, bool automatic)
     }
     const int threads = c->n >= kResidentWideN ? 512 : 256;
     int occ = 0;
-    if (resident_occupancy(c->npad, threads, form, &occ) != cudaSuccess || occ < 1) {
+    const int targets = c->n >= kResidentPairN ? 2 : 1;
+    if (resident_occupancy(c->npad, threads, targets, form, &occ) != cudaSuccess || occ < 1) {
         cudaGetLastError();
         return rp;
     }
     rp.threads = threads;
+    rp.targets = targets;
     rp.form = form;
     // one CTA per SM at most, and at least 8 targets per CTA; an even number of
     // targets per CTA keeps every CTA's staged block a whole number of source pairs
@@ -923,7 +929,7 @@ ResidentPlan compute_resident_plan(const pp_ctx *c, bool automatic)
     rp.grid = (int)((c->n + rp.bt - 1) / rp.bt);
     if (rp.grid > c->sms * occ || rp.grid > kResidentMaxGrid) return rp;
     rp.nsrc = (int)round_up(c->n, 2);
-    const int qmax = threads / rp.bt;
+    const int qmax = threads / (rp.bt / rp.targets);
     // at least 32 sources per thread: fewer partial sums to add at tiny N
     rp.chunk = (int)round_up(std::max((rp.nsrc + qmax - 1) / qmax, std::min(rp.nsrc, 32)), 2);
     rp.q = (rp.nsrc + rp.chunk - 1) / rp.chunk;
@@ -963,6 +969,7 @@ pp_status step_resident(pp_ctx *c, const ResidentPlan &rp, int64_t nsteps)
     ra.stage[1] = c->stage[1];
     ra.bt = rp.bt;
     ra.q = rp.q;
+    ra.targets = rp.targets;
     ra.chunk = rp.chunk;
     ra.nsrc = rp.nsrc;
     ra.flags = c->res_flags;

@@ -114,7 +114,8 @@ struct ResidentArgs {
     int parity0;      // buffer holding the staged r_{n+1} at the first step
     int nsteps;
     int bt;           // targets per CTA (grid = ceil(n / bt))
-    int q;            // threads (source chunks) per target, bt * q <= threads per CTA
+    int targets;      // per thread: 1, or with 512 threads 2
+    int q;            // threads (source chunks) per target, bt / targets * q <= threads per CTA
     int chunk;        // sources per chunk, even
     int nsrc;         // sources summed: n rounded up to even (the odd tail is padding)
     unsigned *flags;  // [0]: grid-barrier arrival counter, zero at launch
@@ -125,9 +126,9 @@ struct ResidentArgs {
 // the plain kernel (the resident kernel folds compensated in every form).
 // bt (targets per CTA) is even.
 enum ResidentForm : int { RES_PLAIN = 0, RES_WEIGHTED = 1, RES_SPLIT = 2, RES_KAHAN = 3 };
-size_t resident_smem(int npad, int threads, int form);
+size_t resident_smem(int npad, int threads, int targets, int form);
 cudaError_t resident_configure(int npad_single, int npad_split);
-cudaError_t resident_occupancy(int npad, int threads, int form, int *blocks_per_sm);
+cudaError_t resident_occupancy(int npad, int threads, int targets, int form, int *blocks_per_sm);
 cudaError_t launch_resident(const ForceArgs &a, const ResidentArgs &ra, int grid, int threads,
                             int form, cudaStream_t stream);
 

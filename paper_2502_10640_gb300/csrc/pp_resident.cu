@@ -111,7 +111,10 @@ __device__ __forceinline__ void push_component(const ForceArgs &p, int i, int c,
 // weight ratio w_j / W (one more f32x2 multiply per two pairs).
 // SPLIT: hi/lo staged positions (STAGE_F32IX2): shared memory holds both
 // parts, and each separation is (hi_i - hi_j) + (lo_i - lo_j).
-template <int NT, bool W, bool SPLIT>
+// R targets per thread.  Two from kResidentPairN on, where with one a source
+// pair's shared-memory loads (two of 16 bytes, four with SPLIT) bound the loop;
+// one below, where twice the partial sums per target cost what the loads save.
+template <int NT, int R, bool W, bool SPLIT>
 __global__ void __launch_bounds__(NT, 1)
     force_resident_kernel(const ForceArgs p, const ResidentArgs ra)
 {
@@ -119,14 +122,15 @@ __global__ void __launch_bounds__(NT, 1)
     float4 *sj4 = reinterpret_cast<float4 *>(smem_raw);   // staged sources, interleaved pairs
     const float *sj = reinterpret_cast<const float *>(smem_raw);
     constexpr int NPARTS = SPLIT ? 2 : 1;                  // hi (and lo) copies, npad each
-    // per-thread partial sums: [hi x, y, z][lo x, y, z] x NT floats
+    // per-thread partial sums: [hi x, y, z][lo x, y, z] x R NT floats
     float *part = reinterpret_cast<float *>(smem_raw + (size_t)NPARTS * p.npad * sizeof(float4));
     __shared__ uint64_t s_bar;   // completion of one step's source copies
     __shared__ int s_abort;
 
     const int tid = threadIdx.x;
-    const int tl = tid % ra.bt, qi = tid / ra.bt;
-    const int i = blockIdx.x * ra.bt + tl;
+    const int per = ra.bt / R;
+    const int tl = tid % per, qi = tid / per;
+    const int i = blockIdx.x * ra.bt + R * tl;   // R = 2: and i + 1 (padding if that is n)
     const bool work = qi < ra.q && i < p.n;
     const int j0 = min(qi * ra.chunk, ra.nsrc), j1 = min(j0 + ra.chunk, ra.nsrc);
     const float eps2 = fmaxf(p.eps2f, kSelfFloor);
@@ -136,7 +140,10 @@ __global__ void __launch_bounds__(NT, 1)
     // Each (component, target) item of the CTA belongs to one thread for the
     // whole launch (3 BT <= threads): that thread alone reads and writes the
     // item's r, v, a, so it keeps them in registers and stores them once at
-    // the end.
+    // the end.  (Tried: four threads per item for the sum.  Adjacent, the owners
+    // spread over more warps and their FP64 instructions, 64 cycles each however
+    // few lanes are active, added 1.1 us per step at N = 4096; a warp apart it
+    // gained 3 % at N = 1000 and nothing above.)
     const int oc = tid / ra.bt, oti = tid - oc * ra.bt;
     const int oi = blockIdx.x * ra.bt + oti;
     const bool owner = tid < 3 * ra.bt && oi < p.n;
@@ -187,66 +194,88 @@ __global__ void __launch_bounds__(NT, 1)
         __syncthreads();
         if (s_abort) return;   // the state is left unspecified (the call reports the timeout)
 
-        float hx = 0.f, hy = 0.f, hz = 0.f, lx = 0.f, ly = 0.f, lz = 0.f;
+        float h[R][3] = {}, l[R][3] = {};
         if (work) {
-            const float *q = sj + 8 * (i >> 1) + (i & 1);
-            const f2_t X = f2_pack(q[0], q[0]), Y = f2_pack(q[2], q[2]), Z = f2_pack(q[4], q[4]);
-            const float *ql = q + 4 * (size_t)p.npad;
-            const f2_t XL = SPLIT ? f2_pack(ql[0], ql[0]) : 0ull;
-            const f2_t YL = SPLIT ? f2_pack(ql[2], ql[2]) : 0ull;
-            const f2_t ZL = SPLIT ? f2_pack(ql[4], ql[4]) : 0ull;
+            f2_t X[R], Y[R], Z[R], XL[R], YL[R], ZL[R];
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const float *q = sj + 8 * ((i + k) >> 1) + ((i + k) & 1);
+                const float *ql = q + 4 * (size_t)p.npad;
+                X[k] = f2_pack(q[0], q[0]);
+                Y[k] = f2_pack(q[2], q[2]);
+                Z[k] = f2_pack(q[4], q[4]);
+                XL[k] = SPLIT ? f2_pack(ql[0], ql[0]) : 0ull;
+                YL[k] = SPLIT ? f2_pack(ql[2], ql[2]) : 0ull;
+                ZL[k] = SPLIT ? f2_pack(ql[4], ql[4]) : 0ull;
+            }
             for (int t0 = j0; t0 < j1; t0 += kResFold) {
                 const int t1 = min(t0 + kResFold, j1);
-                f2_t AX = 0ull, AY = 0ull, AZ = 0ull;
+                f2_t A[R][3] = {};
 #pragma unroll 4
                 for (int j = t0; j < t1; j += 2) {
                     const float4 a = sj4[j];       // x_j x_j+1 y_j y_j+1
                     const float4 b = sj4[j + 1];   // z_j z_j+1 w_j w_j+1
-                    f2_t DX = f2_sub(X, f2_pack(a.x, a.y));
-                    f2_t DY = f2_sub(Y, f2_pack(a.z, a.w));
-                    f2_t DZ = f2_sub(Z, f2_pack(b.x, b.y));
+                    float4 al = make_float4(0.f, 0.f, 0.f, 0.f), bl = al;
                     if (SPLIT) {
-                        const float4 al = sj4[p.npad + j], bl = sj4[p.npad + j + 1];
-                        DX = f2_add(DX, f2_sub(XL, f2_pack(al.x, al.y)));
-                        DY = f2_add(DY, f2_sub(YL, f2_pack(al.z, al.w)));
-                        DZ = f2_add(DZ, f2_sub(ZL, f2_pack(bl.x, bl.y)));
+                        al = sj4[p.npad + j];
+                        bl = sj4[p.npad + j + 1];
                     }
-                    const f2_t S = f2_fma(DZ, DZ, f2_fma(DY, DY, f2_fma(DX, DX, EPS2)));
-                    float s0, s1;
-                    f2_unpack(S, s0, s1);
-                    const f2_t INV = f2_pack(rsqrt_sfu(s0), rsqrt_sfu(s1));
-                    const f2_t INV3 = W ? f2_mul(f2_mul(f2_mul(INV, INV), INV), f2_pack(b.z, b.w))
-                                        : f2_mul(f2_mul(INV, INV), INV);
-                    AX = f2_fma(INV3, DX, AX);
-                    AY = f2_fma(INV3, DY, AY);
-                    AZ = f2_fma(INV3, DZ, AZ);
+#pragma unroll
+                    for (int k = 0; k < R; ++k) {
+                        f2_t DX = f2_sub(X[k], f2_pack(a.x, a.y));
+                        f2_t DY = f2_sub(Y[k], f2_pack(a.z, a.w));
+                        f2_t DZ = f2_sub(Z[k], f2_pack(b.x, b.y));
+                        if (SPLIT) {
+                            DX = f2_add(DX, f2_sub(XL[k], f2_pack(al.x, al.y)));
+                            DY = f2_add(DY, f2_sub(YL[k], f2_pack(al.z, al.w)));
+                            DZ = f2_add(DZ, f2_sub(ZL[k], f2_pack(bl.x, bl.y)));
+                        }
+                        const f2_t S = f2_fma(DZ, DZ, f2_fma(DY, DY, f2_fma(DX, DX, EPS2)));
+                        float s0, s1;
+                        f2_unpack(S, s0, s1);
+                        const f2_t INV = f2_pack(rsqrt_sfu(s0), rsqrt_sfu(s1));
+                        const f2_t INV3 = W ? f2_mul(f2_mul(f2_mul(INV, INV), INV),
+                                                     f2_pack(b.z, b.w))
+                                            : f2_mul(f2_mul(INV, INV), INV);
+                        A[k][0] = f2_fma(INV3, DX, A[k][0]);
+                        A[k][1] = f2_fma(INV3, DY, A[k][1]);
+                        A[k][2] = f2_fma(INV3, DZ, A[k][2]);
+                    }
                 }
-                float x0, x1, y0, y1, z0, z1;
-                f2_unpack(AX, x0, x1);
-                f2_unpack(AY, y0, y1);
-                f2_unpack(AZ, z0, z1);
-                comp_add(hx, lx, x0 + x1);
-                comp_add(hy, ly, y0 + y1);
-                comp_add(hz, lz, z0 + z1);
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        float u, v;
+                        f2_unpack(A[k][c], u, v);
+                        comp_add(h[k][c], l[k][c], u + v);
+                    }
             }
         }
-        part[tid] = hx;
-        part[NT + tid] = hy;
-        part[2 * NT + tid] = hz;
-        part[3 * NT + tid] = lx;
-        part[4 * NT + tid] = ly;
-        part[5 * NT + tid] = lz;
+        // partial t of target R tl + k sits at t * bt + R tl + k (R = 2: one 8-byte store)
+        if (qi < ra.q)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                float *at = part + c * R * NT + qi * ra.bt + R * tl;
+                if (R == 2) {
+                    *reinterpret_cast<float2 *>(at) = make_float2(h[0][c], h[R - 1][c]);
+                    *reinterpret_cast<float2 *>(at + 3 * R * NT) = make_float2(l[0][c], l[R - 1][c]);
+                } else {
+                    at[0] = h[0][c];
+                    at[3 * R * NT] = l[0][c];
+                }
+            }
         __syncthreads();
         // Epilogue, one (component, target) item per thread: the Q partials of
         // the item added with TwoSum in a fixed order, then FP64 for the push.
         if (owner) {
-            float h = 0.f, l = 0.f;
+            float hs = 0.f, ls = 0.f;
             for (int k = 0; k < ra.q; ++k) {
                 const int t = k * ra.bt + oti;
-                comp_add(h, l, part[oc * NT + t]);
-                l = __fadd_rn(l, part[(3 + oc) * NT + t]);
+                comp_add(hs, ls, part[oc * R * NT + t]);
+                ls = __fadd_rn(ls, part[(3 + oc) * R * NT + t]);
             }
-            const double sum = (double)h + (double)l;
+            const double sum = (double)hs + (double)ls;
             push_component<W, SPLIT>(p, oi, oc, occ, sum, r_o, v_o, a_o,
                                      par ? ra.stage[0] : ra.stage[1]);
         }
@@ -266,49 +295,54 @@ __global__ void __launch_bounds__(NT, 1)
     }
 }
 
-template <int NT>
+template <int NT, int R>
 const void *resident_fn_nt(int form)
 {
     switch (form) {
-    case RES_WEIGHTED: return reinterpret_cast<const void *>(&force_resident_kernel<NT, true, false>);
-    case RES_SPLIT: return reinterpret_cast<const void *>(&force_resident_kernel<NT, false, true>);
-    case RES_KAHAN:   // the resident kernel folds compensated in every form
-        return reinterpret_cast<const void *>(&force_resident_kernel<NT, false, false>);
-    default: return reinterpret_cast<const void *>(&force_resident_kernel<NT, false, false>);
+    case RES_WEIGHTED:
+        return reinterpret_cast<const void *>(&force_resident_kernel<NT, R, true, false>);
+    case RES_SPLIT:
+        return reinterpret_cast<const void *>(&force_resident_kernel<NT, R, false, true>);
+    default:   // the resident kernel folds compensated in every form
+        return reinterpret_cast<const void *>(&force_resident_kernel<NT, R, false, false>);
     }
 }
 
-const void *resident_fn(int threads, int form)
+const void *resident_fn(int threads, int targets, int form)
 {
-    return threads == 512 ? resident_fn_nt<512>(form) : resident_fn_nt<256>(form);
+    return threads == 256 ? resident_fn_nt<256, 1>(form)
+           : targets == 2 ? resident_fn_nt<512, 2>(form)
+                          : resident_fn_nt<512, 1>(form);
 }
 
 }  // namespace
 
-size_t resident_smem(int npad, int threads, int form)
+size_t resident_smem(int npad, int threads, int targets, int form)
 {
     return (size_t)(form == RES_SPLIT ? 2 : 1) * npad * sizeof(float4) +
-           6 * (size_t)threads * sizeof(float);
+           6 * (size_t)targets * threads * sizeof(float);
 }
 
 cudaError_t resident_configure(int npad_single, int npad_split)
 {
-    for (int threads : {256, 512})
+    for (int k = 0; k < 3; ++k) {
+        const int threads = k == 0 ? 256 : 512, targets = k == 2 ? 2 : 1;
         for (int form : {RES_PLAIN, RES_WEIGHTED, RES_SPLIT, RES_KAHAN}) {
             const int npad = form == RES_SPLIT ? npad_split : npad_single;
-            cudaError_t e = cudaFuncSetAttribute(resident_fn(threads, form),
+            cudaError_t e = cudaFuncSetAttribute(resident_fn(threads, targets, form),
                                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 (int)resident_smem(npad, threads, form));
+                                                 (int)resident_smem(npad, threads, targets, form));
             if (e != cudaSuccess) return e;
         }
+    }
     return cudaSuccess;
 }
 
-cudaError_t resident_occupancy(int npad, int threads, int form, int *blocks_per_sm)
+cudaError_t resident_occupancy(int npad, int threads, int targets, int form, int *blocks_per_sm)
 {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, resident_fn(threads, form),
-                                                         threads,
-                                                         resident_smem(npad, threads, form));
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        blocks_per_sm, resident_fn(threads, targets, form), threads,
+        resident_smem(npad, threads, targets, form));
 }
 
 cudaError_t launch_resident(const ForceArgs &a, const ResidentArgs &ra, int grid, int threads,
@@ -317,8 +351,9 @@ cudaError_t launch_resident(const ForceArgs &a, const ResidentArgs &ra, int grid
     ForceArgs ca = a;
     ResidentArgs cr = ra;
     void *args[] = {&ca, &cr};
-    return cudaLaunchCooperativeKernel(resident_fn(threads, form), dim3(grid), dim3(threads), args,
-                                       resident_smem(a.npad, threads, form), stream);
+    return cudaLaunchCooperativeKernel(resident_fn(threads, ra.targets, form), dim3(grid),
+                                       dim3(threads), args,
+                                       resident_smem(a.npad, threads, ra.targets, form), stream);
 }
 
 }  // namespace ppk
