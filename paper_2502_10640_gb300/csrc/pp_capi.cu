@@ -152,18 +152,20 @@ constexpr int64_t kBoxGuardWideN = 196608;
 
 // The pair-symmetric kernel (each unordered pair once, pp_sym.cuh) for this
 // context's modes and N, or null where the one-sided kernels are faster.  Its
-// smallest unit of work is a warp's 256 or 512 targets against one tile, so
-// small N leaves too few units; from there on it runs 14 FP32 lane operations
-// per unordered pair instead of 22.  The lines lie where the GB300 sweep has the
-// two level (ms per step, symmetric against one-sided, single staging: 0.104
-// against 0.128 at N = 16384, 0.196 / 0.238 at 24576, 0.315 / 0.407 at 32768,
-// 1.16 / 1.47 at 65536, 4.37 / 5.79 at 131072, 16.8 / 22.5 at 262144; guarded
-// 0.239 / 0.264 at 24576, 1.29 / 1.67 at 65536; on sorted sources 4.64 / 6.13 at
-// 131072, 283 / 366 at 2^20; hi/lo 0.146 / 0.200 at 16384, 27.4 / 33.4 at 262144; weights 0.128 /
-// 0.139 at 16384, 21.2 / 24.3 at 262144).  Tiles of 128 sources below 28672
-// and 256 (512 for single staging) from 196608 on keep the FP32 partial sums no
-// longer than those of the one-sided kernel that would run instead.  Above 2^22
-// the partial sums would pass 18 GB for a step of seconds: one-sided again.
+// smallest unit of work is a warp's 256 or 512 targets against 128 sources, so
+// small N leaves too few units; from there on it runs 14 FP32 lane operations per
+// unordered pair instead of 22.  The lines lie where the GB300 sweep has the two
+// level.  ms per step, symmetric / one-sided:
+//   single    0.118 / 0.129 at N = 16385, 0.202 / 0.241 at 24001, 0.315 / 0.407 at
+//             32768, 1.16 / 1.47 at 65536, 4.37 / 5.79 at 131072, 16.8 / 22.5 at 262144
+//   guarded   0.139 / 0.144 at 16385, 0.239 / 0.256 at 24001, 1.29 / 1.67 at 65536;
+//             on sorted sources 4.64 / 6.13 at 131072, 261 / 366 at 2^20
+//   hi/lo     0.146 / 0.200 at 16384, 1.76 / 2.19 at 65536, 27.4 / 33.4 at 262144
+//   weights   0.127 / 0.139 at 16385, 1.35 / 1.62 at 65536, 21.2 / 24.3 at 262144
+// Tiles of 128 sources below 28672 and 256 (512 for single staging) from 196608 on
+// keep the FP32 partial sums about as long as those of the one-sided kernel that
+// would run instead.  Above 2^22 the partial sums would pass 18 GB for a step of
+// seconds: one-sided again.
 constexpr int64_t kSymMaxN = int64_t(1) << 22;
 const Variant *sym_variant(const pp_ctx *c)
 {
@@ -179,7 +181,7 @@ const Variant *sym_variant(const pp_ctx *c)
                                        : "f32x2split.fold64.sym4k128");
     }
     if (c->positions == PP_POS_GUARDED) {
-        if (n < 20000) return nullptr;
+        if (n < (c->wts ? 20000 : 16384)) return nullptr;
         if (c->wts)
             return variant_by_name(n >= kBoxGuardMinN ? "f32x2wbguard.sfold64.sym8k256"
                                                       : "f32x2wguard.fold64.sym4k128");
@@ -432,6 +434,9 @@ pp_status ensure_sym(pp_ctx *c, const Variant &v, int *at)
         c->sym_ws_bytes = 0;
         if (cudaMalloc(&c->sym_ws, ws) != cudaSuccess) {
             cudaGetLastError();
+            c->sym_ws = nullptr;
+            for (auto &e : c->sym) cudaFree(e.tab);   // plans without partial sums
+            c->sym.clear();
             return fail(PP_ERR_NOMEM, "cannot allocate the partial sums of the symmetric pass");
         }
         c->sym_ws_bytes = ws;
@@ -1625,6 +1630,7 @@ pp_status pp_autotune(pp_ctx *c, pp_tune_result *out)
             vs[v].stage != (c->positions == PP_POS_SPLIT ? STAGE_F32IX2 : STAGE_F32I))
             continue;
         if (vs[v].cluster > 0 && !cluster_fits(vs[v])) continue;   // cannot launch here
+        if (vs[v].sym && (c->sym_off || c->n > kSymMaxN)) continue;   // partial sums too large
         c->variant_override = v;
         c->split_override = 0;
         const Plan base = make_plan(c, vs[v].kind);
@@ -1641,6 +1647,10 @@ pp_status pp_autotune(pp_ctx *c, pp_tune_result *out)
             c->split_override = cand[k];
             // one untimed pass, one pass to size the measurement, then the timed passes
             st = force_pass(c, MODE_FIELDS, scratch, nullptr, c->aos);
+            if (st == PP_ERR_NOMEM && vs[v].sym) {   // no room for its partial sums
+                st = PP_OK;
+                break;
+            }
             if (st != PP_OK) break;
             PP_CUDA(cudaEventRecord(e0, c->stream));
             st = force_pass(c, MODE_FIELDS, scratch, nullptr, c->aos);
