@@ -108,14 +108,6 @@ __device__ __forceinline__ float rsqrt_sfu(float x)
     return y;
 }
 
-// Hardware (SFU) approximate reciprocal, denormals flushed.
-__device__ __forceinline__ float rcp_sfu(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // ---- thread-block clusters (distributed shared memory) ----
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {

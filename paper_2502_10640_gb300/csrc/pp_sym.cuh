@@ -335,7 +335,7 @@ __device__ __forceinline__ void sym_collect(const ForceArgs &p, const SymArgs &q
 // parts alone.  BOX: the caller has ruled close pairs out.  Not inlined: the loop needs every register for
 // itself (inlined into the queue loop it ran 10 % slower).
 template <int PK, int TJ, int WI, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, bool ADD,
-          int RCP, int MINB>
+          int MINB>
 __device__ __noinline__ bool sym_tile(const float *__restrict__ src, size_t lo_at, int n, int i0,
                                       int j0, int count, float eps2, double *acc, int at0, float *stash)
 {
@@ -420,12 +420,7 @@ __device__ __noinline__ bool sym_tile(const float *__restrict__ src, size_t lo_a
                     }
                     if (GUARD) ms[k] = fmax3(ms[k], q0, q1);
                     const f2_t INV = f2_pack(q0, q1);
-                    // RCP: 1/s from the SFU, which has slots left, instead of a product (not
-                    // with OWN, whose self pair has s = 0 without softening)
-                    const f2_t INV2 = !OWN && (RCP == 2 || (RCP == 1 && k % 2 == 1))
-                                          ? f2_pack(rcp_sfu(s0), rcp_sfu(s1))
-                                          : f2_mul(INV, INV);
-                    const f2_t INV3 = f2_mul(INV2, INV);
+                    const f2_t INV3 = f2_mul(f2_mul(INV, INV), INV);
                     const f2_t TI = WEIGHTED ? f2_mul(INV3, WJ) : INV3;
                     A[k][0] = f2_fma(TI, DX, A[k][0]);
                     A[k][1] = f2_fma(TI, DY, A[k][1]);
@@ -485,11 +480,11 @@ __device__ __forceinline__ void sym_split(const float *src, size_t lo_at, int n,
 {
     constexpr int PH = PK > 4 ? 4 : PK;
     static_assert(PK == PH || PK == 2 * PH, "one or two parts");
-    if (!sym_tile<PH, TJ, WI, POS_SPLIT, false, WEIGHTED, KAHAN, OWN, false, 0, MINB>(
+    if (!sym_tile<PH, TJ, WI, POS_SPLIT, false, WEIGHTED, KAHAN, OWN, false, MINB>(
             src, lo_at, n, i0, j0, count, eps2, acc, 0, stash))
         sym_slow<PH, TJ, WI, true, WEIGHTED, KAHAN, OWN>(src, lo_at, n, i0, j0, count, eps2, acc, 0, stash,
                                                         false, true);
-    if (PK > PH && !sym_tile<PH, TJ, WI, POS_SPLIT, false, WEIGHTED, KAHAN, OWN, true, 0, MINB>(
+    if (PK > PH && !sym_tile<PH, TJ, WI, POS_SPLIT, false, WEIGHTED, KAHAN, OWN, true, MINB>(
                        src, lo_at, n, i0 + 64 * PH, j0, count, eps2, acc, 64 * PH, stash)) {
         // the first part's share of the source sums again, then this part
         if (!OWN)
@@ -502,13 +497,13 @@ __device__ __forceinline__ void sym_split(const float *src, size_t lo_at, int n,
 
 // One (warp, tile) by whichever of the forms above it needs.  close: BOX found
 // that it may hold close pairs.
-template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, int RCP, int MINB>
+template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, int MINB>
 __device__ __forceinline__ void sym_any(const float *src, size_t lo_at, int n, int i0, int j0,
                                         int count, float eps2, double *acc, float *stash, bool close)
 {
     constexpr int WI = 64 * PK;
     if (!(BOX && close) &&
-        sym_tile<PK, TJ, WI, POS, BOX, WEIGHTED, KAHAN, OWN, false, RCP, MINB>(
+        sym_tile<PK, TJ, WI, POS, BOX, WEIGHTED, KAHAN, OWN, false, MINB>(
             src, lo_at, n, i0, j0, count, eps2, acc, 0, stash))
         return;
     if (POS == POS_GUARDED)
@@ -549,7 +544,7 @@ __device__ __forceinline__ bool sym_box_close(const float4 *boxes, int t, float4
 // BOX, on spatially sorted sources: a tile whose box comes that close to the
 // box of one of the block's own tiles, and the targets' own tiles, are summed on hi/lo parts,
 // every other tile on hi parts with no test per pair.
-template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, int MINB, int RCP>
+template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, int MINB>
 __global__ void __launch_bounds__(kSymThreads, MINB)
     force_sym_kernel(const ForceArgs p, const SymArgs q)
 {
@@ -597,10 +592,10 @@ __global__ void __launch_bounds__(kSymThreads, MINB)
                 const bool mine = j < i0 + WI;   // the sources are among the targets
                 len = min(TJ - j % TJ, it.j1 - j);
                 if (mine)
-                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, true, RCP, MINB>(
+                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, true, MINB>(
                         src, lo_at, p.n, i0, j, len, p.eps2f, acc, stash, true);
                 else
-                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, false, RCP, MINB>(
+                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, false, MINB>(
                         src, lo_at, p.n, i0, j, len, p.eps2f, acc, stash,
                         BOX && __any_sync(0xffffffffu, sym_box_close(p.boxes, j / TJ, lo, hi, rmax2,
                                                                      p.eps2f)));
