@@ -235,6 +235,7 @@ __device__ __noinline__ void sym_slow(const float *__restrict__ src, size_t lo_a
         for (int g = 0; g < G; ++g)
             if (fold) sym_fold<WI, KAHAN>(acc, at0 + (p + g) * 64 + 2 * lane, A[g]);
     }
+    __syncwarp();   // sym_tile with ADD reads the stash in other lanes
 }
 
 // Add the partial sums of 32 particles and run their push.  The order of the
@@ -619,6 +620,7 @@ __global__ void __launch_bounds__(kSymThreads, MINB)
                             __stcg(out + c * plane + s + 32 * h, v[h][c]);
                         }
                 }
+                __syncwarp();   // the next tile's sums enter the stash in other lanes
             }
             // this item's sums of the block's targets, each written by its owner
             double *part = q.ipart + ((size_t)item * q.ki + kb) * 3 * WI;
