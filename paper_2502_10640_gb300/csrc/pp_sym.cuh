@@ -146,8 +146,18 @@ __device__ __forceinline__ void load_lows(const float *lo, int i, int n, f2_t &x
     }
 }
 
-// The slow form of one (warp, tile): zero-distance pairs skipped, separations
-// on hi/lo parts with SPLIT, two packs at a time so that it needs few
+// v with the lanes that are not `on` set to 0.
+__device__ __forceinline__ f2_t f2_keep(f2_t v, bool on0, bool on1)
+{
+    float a, b;
+    f2_unpack(v, a, b);
+    return f2_pack(on0 ? a : 0.f, on1 ? b : 0.f);
+}
+
+// The slow form of one (warp, tile): pairs with s == 0 or s not a number add
+// nothing (their separation is dropped with the factor: 0 * NaN would stay in both
+// sums, and one particle lost in a close encounter would take the bunch with it),
+// separations on hi/lo parts with SPLIT, two packs at a time so that it needs few
 // registers.  Arguments as sym_tile; fold = false leaves the targets' sums alone.
 template <int PK, int TJ, int WI, bool SPLIT, bool WEIGHTED, bool KAHAN, bool OWN>
 __device__ __noinline__ void sym_slow(const float *__restrict__ src, size_t lo_at, int n, int i0,
@@ -191,8 +201,11 @@ __device__ __noinline__ void sym_slow(const float *__restrict__ src, size_t lo_a
                     const f2_t S = f2_fma(DZ, DZ, f2_fma(DY, DY, f2_fma(DX, DX, EPS2)));
                     float s0, s1;
                     f2_unpack(S, s0, s1);
-                    const f2_t INV = f2_pack(s0 > 0.f ? rsqrt_sfu(s0) : 0.f,
-                                             s1 > 0.f ? rsqrt_sfu(s1) : 0.f);
+                    const bool on0 = s0 > 0.f, on1 = s1 > 0.f;
+                    const f2_t INV = f2_pack(on0 ? rsqrt_sfu(s0) : 0.f, on1 ? rsqrt_sfu(s1) : 0.f);
+                    DX = f2_keep(DX, on0, on1);
+                    DY = f2_keep(DY, on0, on1);
+                    DZ = f2_keep(DZ, on0, on1);
                     const f2_t INV3 = f2_mul(f2_mul(INV, INV), INV);
                     const f2_t TI = WEIGHTED ? f2_mul(INV3, f2_pack(wj, wj)) : INV3;
                     A[g][0] = f2_fma(TI, DX, A[g][0]);

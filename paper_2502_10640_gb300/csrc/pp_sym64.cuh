@@ -69,9 +69,16 @@ __global__ void __launch_bounds__(kSymThreads, kSym64Ctas)
 #pragma unroll 1
                 for (int r = 0; r < 32; ++r) {
                     const int jr = j + ((lane + r) & 31);
-                    const double dx = t.x - s.x, dy = t.y - s.y, dz = t.z - s.z;
+                    double dx = t.x - s.x, dy = t.y - s.y, dz = t.z - s.z;
                     const double d2 = fma(dz, dz, fma(dy, dy, fma(dx, dx, p.eps2d)));
-                    const bool on = __double_as_longlong(d2) != 0 && jr < p.n && real && jr != i;
+                    // 0 < d2 <= inf by its bits; a pair with d2 not a number adds nothing at
+                    // all (0 * NaN would stay in both sums)
+                    const bool some = (unsigned long long)__double_as_longlong(d2) - 1ull <
+                                      0x7ff0000000000000ull;
+                    const bool on = some && jr < p.n && real && jr != i;
+                    dx = some ? dx : 0.0;
+                    dy = some ? dy : 0.0;
+                    dz = some ? dz : 0.0;
                     double c = inv_cube_root2(d2);
                     c = on ? c : 0.0;
                     const double ci = WEIGHTED ? c * s.w : c;
