@@ -26,7 +26,7 @@ namespace ppk {
 
 constexpr int kSym64Targets = 32, kSym64Unit = 32, kSym64Ctas = 2;
 
-// s^(-3/2) for s > 0.
+// s^(-3/2) for 0 < s <= inf.
 __device__ __forceinline__ double inv_cube_root2(double s)
 {
     double y;
@@ -34,7 +34,10 @@ __device__ __forceinline__ double inv_cube_root2(double s)
     const double t = y * y;   // y has at most 21 significant bits: exact
     const double e = fma(-s, t, 1.0);
     const double y3 = y * t;
-    return fma(y3 * e, fma(1.875, e, 1.5), y3);
+    const double c = fma(y3 * e, fma(1.875, e, 1.5), y3);
+    // at the ends of the range the series would give inf - inf or 0 * NaN: s below 1e-205
+    // has y3 = inf, s = inf has y3 = 0 (tested by its bits)
+    return (unsigned long long)__double_as_longlong(y3) - 1ull < 0x7fefffffffffffffull ? c : y3;
 }
 
 template <bool WEIGHTED>
