@@ -125,8 +125,9 @@ typedef enum {
 enum {
     PP_OPT_ACC = 1,            /* value: a pp_acc                                              */
     PP_OPT_STREAM = 2,         /* value: cudaStream_t cast to int64 (0 = the context's own)   */
-    PP_OPT_SPLIT = 3,          /* value: j-split count S >= 1 (pair-symmetric kernels: ranges a
-                                  row of tiles is cut into), or 0 for automatic              */
+    PP_OPT_SPLIT = 3,          /* value: j-split count S >= 1 (pair-symmetric kernels: ranges of
+                                  at most N / S sources, never longer than the automatic
+                                  ones), or 0 for automatic                                  */
     PP_OPT_GRAPH_BLOCK = 4,    /* value: steps per captured CUDA graph (0 = plain launches)   */
     PP_OPT_TIMEOUT_NS = 5,     /* value: limit of each device-side wait in ns (default 1e9, or
                                   the environment variable PP_TIMEOUT_NS at creation)        */

@@ -415,9 +415,10 @@ pp_status ensure_sym(pp_ctx *c, const Variant &v, int *at)
             return PP_OK;
         }
     const int64_t slots = (int64_t)c->sms * resident_ctas(v);
-    const SymPlan sp = make_sym_plan((int)c->n, c->npad, v, slots, c->split_override);
+    const SymPlan sp = make_sym_plan((int)c->n, c->npad, 32 * v.R, v.kind == KIND_FORCE64, slots,
+                                     c->split_override);
     const size_t ib = round_up(sp.items.size() * sizeof(SymItem), 256);
-    const size_t rb = round_up(sp.rows.size() * sizeof(int2), 256);
+    const size_t rb = round_up(sp.rows.size() * sizeof(SymRow), 256);
     const size_t ws = (sp.row_doubles + sp.part_doubles) * sizeof(double);
     // a pass with the old buffers may be running, or captured in a graph
     if (ws > c->sym_ws_bytes || c->sym.size() >= kSymPlans) {
@@ -450,7 +451,7 @@ pp_status ensure_sym(pp_ctx *c, const Variant &v, int *at)
     unsigned char *t = static_cast<unsigned char *>(e.tab);
     if (cudaMemcpyAsync(t, sp.items.data(), sp.items.size() * sizeof(SymItem),
                         cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
-        cudaMemcpyAsync(t + ib, sp.rows.data(), sp.rows.size() * sizeof(int2),
+        cudaMemcpyAsync(t + ib, sp.rows.data(), sp.rows.size() * sizeof(SymRow),
                         cudaMemcpyHostToDevice, c->stream) != cudaSuccess ||
         cudaMemsetAsync(t + ib + rb, 0, 256, c->stream) != cudaSuccess ||
         cudaStreamSynchronize(c->stream) != cudaSuccess) {   // the host tables end with this call
@@ -458,7 +459,7 @@ pp_status ensure_sym(pp_ctx *c, const Variant &v, int *at)
         return cuda_fail(cudaGetLastError(), "work-item tables");
     }
     e.args.items = reinterpret_cast<const SymItem *>(t);
-    e.args.rows = reinterpret_cast<const int2 *>(t + ib);
+    e.args.rows = reinterpret_cast<const SymRow *>(t + ib);
     e.args.ctl = reinterpret_cast<unsigned *>(t + ib + rb);
     e.args.nitems = (int)sp.items.size();
     e.args.ki = sp.ki;

@@ -87,19 +87,9 @@ void set_last_error(const char *msg);
 // Table of compiled force-kernel variants.
 const Variant *variants(int *count);
 
-// Pair-symmetric kernels (pp_sym.cu): their table entries, the work plan of one
-// pass (host arrays; the caller keeps device copies) and the launcher.
-// Partial-sum rows: at most this many groups of target blocks, so the rows take
-// at most 12 * kSymMaxRows bytes per particle.
-constexpr int kSymMaxRows = 128;
-struct SymPlan {
-    int ki = 1;
-    std::vector<SymItem> items;
-    std::vector<int2> rows;
-    size_t row_doubles = 0, part_doubles = 0;
-};
+// Pair-symmetric kernels (pp_sym.cu): their table entries and the launcher.  The
+// work plan of a pass is in pp_sym_plan.h (host arrays; the caller keeps device copies).
 std::vector<Variant> sym_variants();
-SymPlan make_sym_plan(int n, int npad, const Variant &v, int64_t slots, int split);
 cudaError_t launch_sym(const Variant &v, const ForceArgs &a, const SymArgs &q, int grid,
                        cudaStream_t stream);
 

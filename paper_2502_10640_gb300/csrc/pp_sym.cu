@@ -1,7 +1,5 @@
-// pp_sym.cu -- instantiations, work plan and launcher of the pair-symmetric
-// force kernels (pp_sym.cuh).
-#include <algorithm>
-
+// pp_sym.cu -- instantiations and launcher of the pair-symmetric force kernels
+// (pp_sym.cuh; the work plan is in pp_sym_plan.h).
 #include "pp_internal.h"
 #include "pp_sym64.cuh"
 
@@ -65,48 +63,6 @@ std::vector<Variant> sym_variants()
         make_sym64<false>("f64.full.symr1k32"),
         make_sym64<true>("f64w.full.symr1k32"),
     };
-}
-
-// Work items of one pass: each group of ki target blocks walks the sources from
-// its own start to the end; its row is cut into ranges of half a resident warp's
-// share of the remaining work (at most a quarter of its share of the whole: the
-// warps of a scheduler do not advance evenly, with whole shares at the start the
-// pass took 40 % longer), long ranges first, so the tail of the pass is short.
-// The shortest range is 128 sources, 256 where that leaves two to four rounds
-// of items (ms per step, 128 against 256: 0.104 / 0.152 at N = 16384, 0.213 /
-// 0.196 at 24576, 0.339 / 0.315 at 32768, 1.16 / 1.17 at 65536).  split > 0 cuts
-// every row into npad / split.  Each item keeps its own sums, which bounds how
-// finely the work may be cut: rows and items take 5 KB per particle at 2^20.
-SymPlan make_sym_plan(int n, int npad, const Variant &v, int64_t slots, int split)
-{
-    SymPlan pl;
-    const bool f64 = v.kind == KIND_FORCE64;
-    const int WI = 32 * v.R, unit = f64 ? kSym64Unit : kSymUnit, BU = WI / unit, nu = npad / unit;
-    const int nib = (n + WI - 1) / WI;
-    // the rows of partial sums take 24 bytes x npad x groups / 2
-    pl.ki = std::max(1, (nib + kSymMaxRows - 1) / kSymMaxRows);
-    const int groups = (nib + pl.ki - 1) / pl.ki;
-    double left = 0.0;
-    for (int g = 0; g < groups; ++g)
-        left += (double)std::min(pl.ki, nib - g * pl.ki) * (nu - g * pl.ki * BU);
-    const double warps = kSymWarps * (double)slots, most = left / (4.0 * warps);
-    const int least = f64 ? 1 : n >= 20480 && n < 40960 ? 4 : 2;
-    for (int g = 0; g < groups; ++g) {
-        const int ib0 = g * pl.ki, nb = std::min(pl.ki, nib - ib0);
-        const int first = (int)pl.items.size();
-        for (int u = ib0 * BU; u < nu;) {
-            int len = split > 0 ? (nu + split - 1) / split
-                                : (int)(std::min(left / (2.0 * warps), most) / nb);
-            len = std::max(1, std::min(std::max(len, split > 0 ? 1 : least), nu - u));
-            pl.items.push_back(SymItem{ib0, nb, u * unit, (u + len) * unit});
-            left -= (double)nb * len;
-            u += len;
-        }
-        pl.rows.push_back(make_int2(first, (int)pl.items.size() - first));
-    }
-    pl.row_doubles = sym_row_offset(groups, npad, pl.ki * WI);
-    pl.part_doubles = pl.items.size() * pl.ki * 3 * (size_t)WI;
-    return pl;
 }
 
 cudaError_t launch_sym(const Variant &v, const ForceArgs &a, const SymArgs &q, int grid,

@@ -32,15 +32,9 @@
 #pragma once
 
 #include "pp_force.cuh"
+#include "pp_sym_plan.h"
 
 namespace ppk {
-
-// One item of work: target blocks [ib0, ib0 + nb) against sources [j0, j1)
-// (multiples of kSymUnit).
-struct SymItem {
-    int ib0, nb, j0, j1;
-};
-constexpr int kSymUnit = 64;
 
 // The queue words of a pass, zero between launches (the last CTA to leave
 // clears them).
@@ -48,22 +42,13 @@ enum SymCtl : int { SYM_NEXT = 0, SYM_DONE = 1, SYM_FINISH = 2, SYM_LEFT = 3, SY
 
 struct SymArgs {
     const SymItem *items;
-    const int2 *rows;         // per group of ki target blocks: (first item, items)
+    const SymRow *rows;       // per group of ki target blocks
     unsigned *ctl;            // [SYM_CTL]
     double *jrow;             // per group: [3][npad - start] sums over its targets
     double *ipart;            // per (item, block of its group): [3][WI] sums
     int nitems;
     int ki;                   // target blocks per group
 };
-
-// Doubles before the row of group g (rows are packed: row g starts at source g * bis).
-__host__ __device__ __forceinline__ size_t sym_row_offset(int g, int npad, int bis)
-{
-    return 3 * ((size_t)g * npad - (size_t)bis * ((size_t)g * (g - 1) / 2));
-}
-
-constexpr int kSymThreads = 128;
-constexpr int kSymWarps = kSymThreads / 32;
 
 __device__ __forceinline__ f2_t f2_shfl(f2_t v, int from)
 {
@@ -263,10 +248,10 @@ __device__ __forceinline__ void sym_finish(const ForceArgs &p, const SymArgs &q,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int bis = WI * q.ki;
     const int ib = j0 / WI, grp = ib / q.ki;
-    const int2 row = q.rows[grp];
-    const int j = j0 + lane, terms = grp + 1 + row.y;
+    const SymRow row = q.rows[grp];
+    const int j = j0 + lane, terms = grp + 1 + row.items;
     const double *own =
-        q.ipart + ((size_t)row.x * q.ki + (ib - grp * q.ki)) * 3 * WI + (j - ib * WI);
+        q.ipart + ((size_t)row.first * q.ki + (ib - grp * q.ki)) * 3 * WI + (j - ib * WI);
     double sum[3] = {0.0, 0.0, 0.0};
     for (int k0 = warp * U; k0 < terms; k0 += kSymWarps * U) {
         double v[3][U];

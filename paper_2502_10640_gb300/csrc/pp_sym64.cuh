@@ -24,7 +24,7 @@
 
 namespace ppk {
 
-constexpr int kSym64Targets = 32, kSym64Unit = 32, kSym64Ctas = 2;
+constexpr int kSym64Targets = 32, kSym64Ctas = 2;
 
 // s^(-3/2) for 0 < s <= inf.
 __device__ __forceinline__ double inv_cube_root2(double s)

@@ -1,0 +1,95 @@
+"""The work plan of the pair-symmetric passes (csrc/pp_sym_plan.h, host code), checked by a
+small C++ program: every source of every row is covered once, and no item of work is longer
+than half a warp's share of what is left when it is handed out, whatever PP_OPT_SPLIT says
+(the warps of a pass wait, bounded, for its last item)."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+from paper_2502_10640_gb300 import build
+
+DRIVER = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "pp_sym_plan.h"
+using namespace ppk;
+// argv: (n, targets, f64, slots, split)...; prints per plan: items, covered, over, longest
+int main(int argc, char **argv)
+{
+    for (int a = 1; a + 4 < argc; a += 5) {
+        const int n = atoi(argv[a]), targets = atoi(argv[a + 1]), f64 = atoi(argv[a + 2]);
+        const int slots = atoi(argv[a + 3]), split = atoi(argv[a + 4]);
+        const int npad = (n + 1023) / 1024 * 1024, unit = f64 ? kSym64Unit : kSymUnit;
+        const SymPlan p = make_sym_plan(n, npad, targets, f64 != 0, slots, split);
+        const double warps = 4.0 * slots;
+        double left = 0.0, longest = 0.0, over = 0.0;
+        for (const SymItem &i : p.items) left += (double)i.nb * (i.j1 - i.j0);
+        const double total = left;
+        size_t at = 0;
+        bool ok = true;
+        int blocks = 0;
+        for (size_t g = 0; g < p.rows.size(); ++g) {
+            ok &= p.rows[g].first == (int)at;
+            int j = -1;
+            for (int k = 0; k < p.rows[g].items; ++k, ++at) {
+                const SymItem &i = p.items[at];
+                if (k == 0) {
+                    ok &= i.ib0 == blocks && i.j0 == i.ib0 * targets;
+                    blocks += i.nb;
+                } else {
+                    ok &= i.j0 == j && i.ib0 == p.items[at - 1].ib0 && i.nb == p.items[at - 1].nb;
+                }
+                ok &= i.j1 > i.j0 && i.j0 % unit == 0 && i.j1 % unit == 0;
+                j = i.j1;
+                const double len = (double)i.nb * (i.j1 - i.j0);
+                // the shortest range is 256 sources (one unit with FP64)
+                const double fair = left / (2.0 * warps), floor_ = (double)i.nb * (f64 ? unit : 256);
+                over = std::max(over, len - std::max(fair, floor_));
+                longest = std::max(longest, len);
+                left -= len;
+            }
+            ok &= j == npad;
+        }
+        ok &= blocks == (n + targets - 1) / targets && at == p.items.size();
+        ok &= p.part_doubles == p.items.size() * p.ki * 3 * (size_t)targets;
+        printf("%zu %d %.6g %.6g\n", p.items.size(), (int)ok, over / total, longest / total);
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def driver(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    d = tmp_path_factory.mktemp("plan")
+    src = d / "plan.cpp"
+    src.write_text(DRIVER)
+    exe = str(d / "plan")
+    subprocess.run([cxx, "-std=c++17", "-O1", "-Wall", "-I", build.CSRC, str(src), "-o", exe],
+                   check=True)
+
+    def plans(rows):
+        args = [str(v) for r in rows for v in r]
+        out = subprocess.run([exe, *args], check=True, capture_output=True, text=True).stdout
+        return [(int(a), int(b), float(c), float(e)) for a, b, c, e in
+                (line.split() for line in out.splitlines())]
+    return plans
+
+
+@pytest.mark.parametrize("n,targets,f64,slots", [
+    (1 << 22, 512, 0, 456), (1 << 20, 512, 0, 456), ((1 << 20) - 77, 512, 0, 304),
+    (1 << 20, 256, 0, 608), (100003, 512, 0, 456), (24001, 256, 0, 608), (14336, 256, 0, 456),
+    (1, 256, 0, 456), (1 << 22, 32, 1, 304), (1 << 20, 32, 1, 304), (131072, 32, 1, 304),
+    (16385, 32, 1, 304), (1, 32, 1, 304)])
+def test_no_item_outlasts_the_pass_whatever_the_split(driver, n, targets, f64, slots):
+    splits = (0, 1, 2, 3, 7, 64, 4096)
+    got = driver([(n, targets, f64, slots, s) for s in splits])
+    for s, (items, covered, over, longest) in zip(splits, got):
+        assert covered == 1, s
+        assert over <= 1e-12, s                 # of the pass's whole work
+        assert longest <= got[0][3], s          # a split only shortens the ranges
+        assert items >= got[0][0], s
