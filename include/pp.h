@@ -130,7 +130,10 @@ enum {
                                   ones), or 0 for automatic                                  */
     PP_OPT_GRAPH_BLOCK = 4,    /* value: steps per captured CUDA graph (0 = plain launches)   */
     PP_OPT_TIMEOUT_NS = 5,     /* value: limit of each device-side wait in ns (default 1e9, or
-                                  the environment variable PP_TIMEOUT_NS at creation)        */
+                                  the environment variable PP_TIMEOUT_NS at creation).  The
+                                  pair-symmetric kernels' wait for the pass's last items of
+                                  work, which run up to some 50 ms at the largest N, takes a
+                                  limit below 1e9 as 1e9                                     */
     PP_OPT_VARIANT = 6,        /* value: force-kernel variant index (-1 = automatic)          */
     PP_OPT_POSITIONS = 7,      /* value: a pp_positions (FP32 pair paths only)                 */
     PP_OPT_RESIDENT = 8,       /* value: a pp_resident (small-N stepping)                      */
@@ -140,7 +143,9 @@ enum {
                                   pass or step (1, or 1 + the spatial sort's with the tile-box
                                   guard of PP_POS_GUARDED)                                   */
     PP_OPT_TEST_SKIP_COPY = 99 /* value: 1 = the next force launch withholds one tile copy (the
-                                  resident kernel: CTA 0's first barrier arrival), so its bounded
+                                  resident kernel: CTA 0's first barrier arrival; the
+                                  pair-symmetric kernels: the completion of one item, with
+                                  PP_OPT_TIMEOUT_NS as set), so its bounded
                                   waits expire and the call returns PP_ERR_TIMEOUT (tests the
                                   timeout path; no fault, no hang) */
 };

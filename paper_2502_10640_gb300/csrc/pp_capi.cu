@@ -350,11 +350,10 @@ struct Plan {
 
 // Choose S, the number of j-chunks per i-block, to fill the GPU: minimise
 // (waves of CTAs) x (tiles per CTA + fixed per-CTA overhead).
-Plan make_plan(pp_ctx *c, int kind, bool one_sided = false)
+Plan make_plan(pp_ctx *c, int kind)
 {
     Plan pl{};
     pl.v = pick_variant(c, kind);
-    if (one_sided && pl.v->sym) pl.v = one_sided_variant(c);
     const int BI = pl.v->T * pl.v->R;
     pl.nib = (int)((c->n + BI - 1) / BI);
     pl.nipad = pl.nib * BI;
@@ -607,14 +606,14 @@ cudaError_t launch_force(pp_ctx *c, const Plan &pl, ForceArgs a)
 // The plan of a pass with its workspaces.  Where the default plan is symmetric
 // and its partial sums cannot be allocated, the context goes on with the
 // one-sided kernels.
-pp_status plan_pass(pp_ctx *c, int kind, bool one_sided, Plan *pl)
+pp_status plan_pass(pp_ctx *c, int kind, Plan *pl)
 {
-    *pl = make_plan(c, kind, one_sided);
+    *pl = make_plan(c, kind);
     pp_status st = ensure_workspace(c, *pl);
     if (st == PP_ERR_NOMEM && pl->v->sym && pl->v == sym_variant(c)) {
         c->sym_off = true;
         drop_graphs(c);
-        *pl = make_plan(c, kind, one_sided);
+        *pl = make_plan(c, kind);
         st = ensure_workspace(c, *pl);
     }
     return st;
@@ -624,9 +623,8 @@ pp_status plan_pass(pp_ctx *c, int kind, bool one_sided, Plan *pl)
 pp_status force_pass(pp_ctx *c, int mode, const void *src, void *dst, double *out)
 {
     const int kind = f64_pairs(c) ? KIND_FORCE64 : KIND_FORCE32;
-    // the symmetric kernels make no tile copies: the test hook takes a one-sided one
     Plan pl{};
-    pp_status st = plan_pass(c, kind, c->skip_copy != 0, &pl);
+    pp_status st = plan_pass(c, kind, &pl);
     if (st != PP_OK) return st;
     ForceArgs a = base_args(c, pl, mode, src, dst, out);
     a.skip_copy = c->skip_copy;
@@ -830,7 +828,7 @@ pp_status build_graphs(pp_ctx *c)
     drop_graphs(c);
     const int kind = f64_pairs(c) ? KIND_FORCE64 : KIND_FORCE32;
     Plan pl{};
-    pp_status st = plan_pass(c, kind, false, &pl);
+    pp_status st = plan_pass(c, kind, &pl);
     if (st != PP_OK) return st;
     for (int p0 = 0; p0 < 2; ++p0) {
         cudaGraph_t g = nullptr;

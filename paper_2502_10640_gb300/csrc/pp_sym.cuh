@@ -40,6 +40,9 @@ namespace ppk {
 // clears them).
 enum SymCtl : int { SYM_NEXT = 0, SYM_DONE = 1, SYM_FINISH = 2, SYM_LEFT = 3, SYM_CTL = 4 };
 
+// Least limit of the wait for a pass's last items (sym_collect).
+constexpr uint64_t kSymMinWaitNs = 1000000000ull;
+
 struct SymArgs {
     const SymItem *items;
     const SymRow *rows;       // per group of ki target blocks
@@ -295,15 +298,18 @@ __device__ __forceinline__ void sym_collect(const ForceArgs &p, const SymArgs &q
     __syncwarp();
     if (lane == 0) atomicAdd(&q.ctl[SYM_DONE], (unsigned)done);
 
-    // Every item has been handed out, each to a warp that runs now: wait (bounded, by at
-    // least a second: it covers the other warps' last items) until all are done, then
-    // share out the particles.
+    // Every item has been handed out, each to a warp that runs now: wait until all are
+    // done, then share out the particles.  The wait covers the other warps' last items
+    // (up to 50 ms at the largest N), so it is bounded by at least a second.  Test hook
+    // (PP_OPT_TEST_SKIP_COPY): wait for one item more than there are, by the limit as set.
     __syncthreads();
     if (tid == 0) {
         int ok = 1;
         const uint64_t t0 = globaltimer_ns();
-        const uint64_t limit = p.timeout_ns > 1000000000ull ? p.timeout_ns : 1000000000ull;
-        while (ld_acquire(&q.ctl[SYM_DONE]) < (unsigned)q.nitems)
+        const uint64_t limit =
+            p.skip_copy || p.timeout_ns > kSymMinWaitNs ? p.timeout_ns : kSymMinWaitNs;
+        const unsigned want = (unsigned)q.nitems + (p.skip_copy ? 1u : 0u);
+        while (ld_acquire(&q.ctl[SYM_DONE]) < want)
             if (globaltimer_ns() - t0 > limit) {
                 ok = 0;
                 break;
