@@ -53,9 +53,15 @@ struct SymPlan {
 // remaining work (at most a quarter of its share of the whole: the warps of a
 // scheduler do not advance evenly, with whole shares at the start the pass took
 // 40 % longer), long ranges first, so the tail of the pass is short.
-// The shortest range is 128 sources, 256 where that leaves two to four rounds
-// of items (ms per step, 128 against 256: 0.104 / 0.152 at N = 16384, 0.213 /
-// 0.196 at 24576, 0.339 / 0.315 at 32768, 1.16 / 1.17 at 65536).
+// The shortest range (`least`) is chosen by the units of work per resident warp, r:
+// 64 sources where 128 would leave fewer than 1.6 rounds of items, 256 where that
+// leaves about two to three and a half, else 128 (one long item too many costs a whole
+// round; above, ranges hardly matter).  ms per step with 64 / 128 / 256 sources:
+//   r = 2.3  hi/lo   N = 13001  0.112 / 0.142 / 0.147      2.6  guarded 14336  0.109 / 0.123 / 0.160
+//   r = 3.5  single  14336      0.099 / 0.090 / 0.127      5.1  single  16385  0.145 / 0.123 / 0.163
+//   r = 5.9  guarded 20481      0.201 / 0.184 / 0.225      7.0  weights 22529  0.247 / 0.228 / 0.238
+//   r = 7.7  guarded 24576      0.260 / 0.243 / 0.234      9.1  Kahan   32768  0.366 / 0.353 / 0.326
+//   r = 13.6 weights 32768      0.396 / 0.391 / 0.373     17.6  weights 36865  0.524 / 0.520 / 0.528
 // split > 0 shortens the ranges to npad / split where they are longer; it never
 // lengthens them, since the warps without work wait for the last item, and a row
 // on one warp takes seconds at N = 2^20.  Each item keeps its own sums, which
@@ -73,7 +79,8 @@ inline SymPlan make_sym_plan(int n, int npad, int targets, bool f64, int64_t slo
     for (int g = 0; g < groups; ++g)
         left += (double)std::min(pl.ki, nib - g * pl.ki) * (nu - g * pl.ki * BU);
     const double warps = kSymWarps * (double)slots, most = left / (4.0 * warps);
-    const int least = f64 ? 1 : n >= 20480 && n < 40960 ? 4 : 2;
+    const double r = left / warps;
+    const int least = f64 || r < 3.2 ? 1 : r >= 7.4 && r < 14.0 ? 4 : 2;
     const int cap = split > 0 ? std::max(1, (nu + split - 1) / split) : nu;
     for (int g = 0; g < groups; ++g) {
         const int ib0 = g * pl.ki, nb = std::min(pl.ki, nib - ib0);
