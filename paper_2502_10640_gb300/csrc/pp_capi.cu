@@ -152,20 +152,27 @@ constexpr int64_t kBoxGuardWideN = 196608;
 
 // The pair-symmetric kernel (each unordered pair once, pp_sym.cuh) for this
 // context's modes and N, or null where the one-sided kernels are faster.  Its
-// smallest unit of work is a warp's 256 or 512 targets against 128 sources, so
+// smallest unit of work is a warp's 256 or 512 targets against 64 to 256 sources, so
 // small N leaves too few units; from there on it runs 14 FP32 lane operations per
 // unordered pair instead of 22.  The lines lie where the GB300 sweep has the two
 // level.  ms per step, symmetric / one-sided:
-//   single    0.118 / 0.129 at N = 16385, 0.202 / 0.241 at 24001, 0.315 / 0.407 at
-//             32768, 1.16 / 1.47 at 65536, 4.37 / 5.79 at 131072, 16.8 / 22.5 at 262144
-//   guarded   0.139 / 0.144 at 16385, 0.239 / 0.256 at 24001, 1.29 / 1.67 at 65536;
-//             on sorted sources 4.64 / 6.13 at 131072, 261 / 366 at 2^20
-//   hi/lo     0.146 / 0.200 at 16384, 1.76 / 2.19 at 65536, 27.4 / 33.4 at 262144
-//   weights   0.127 / 0.139 at 16385, 1.35 / 1.62 at 65536, 21.2 / 24.3 at 262144
-// Tiles of 128 sources below 28672 and 256 (512 for single staging) from 196608 on
-// keep the FP32 partial sums about as long as those of the one-sided kernel that
-// would run instead.  Above 2^22 the partial sums would pass 18 GB for a step of
-// seconds: one-sided again.
+//   single         0.090 / 0.101 at N = 14336, 0.206 / 0.241 at 24001, 0.341 / 0.407 at
+//                  32768, 1.12 / 1.47 at 65536, 4.37 / 5.79 at 131072, 16.8 / 22.5 at 262144
+//   Kahan          0.106 / 0.099 at 14336, 0.114 / 0.117 at 15361, 0.319 / 0.452 at 32768
+//   weights        0.110 / 0.109 at 14336, 0.128 / 0.128 at 15361, 0.130 / 0.139 at 16385,
+//                  0.397 / 0.496 at 32768, 1.27 / 1.62 at 65536, 21.2 / 24.3 at 262144
+//   guarded        0.128 / 0.124 at 15361, 0.130 / 0.139 at 16384, 0.358 / 0.448 at 32768,
+//                  1.26 / 1.66 at 65536; on sorted sources 4.64 / 6.13 at 131072, 260 / 366
+//                  at 2^20; Kahan 0.130 / 0.136 at 16384, weights 0.142 / 0.144
+//   hi/lo          0.112 / 0.163 at 13001, 1.59 / 2.20 at 65536, 27.4 / 33.4 at 262144;
+//                  Kahan 0.114 / 0.163 at 13001, weights 0.108 / 0.166
+// The tiles (64 to 512 sources) keep the FP32 partial sum of a target no longer than
+// that of the one-sided kernel that would run instead: 64 terms below N = 49152 (Kahan
+// and weights 32768, guarded 98304), 128 to 512 above.  Folding every 64 sources costs
+// 8 % at N = 32768, single (0.341 against 0.314 with 256), 0 to 5 % with the blocks of
+// 256 targets.  Those blocks are faster below N = 32768 (Kahan, 28672) and, with the test
+// per pair, at every N (guarded 65536: 1.26 against 1.30 with 512).  Above 2^22 the
+// partial sums would pass 18 GB for a step of seconds: one-sided again.
 constexpr int64_t kSymMaxN = int64_t(1) << 22;
 const Variant *sym_variant(const pp_ctx *c)
 {
@@ -181,27 +188,31 @@ const Variant *sym_variant(const pp_ctx *c)
                                        : "f32x2split.fold64.sym4k128");
     }
     if (c->positions == PP_POS_GUARDED) {
-        if (n < (c->wts ? 20000 : 16384)) return nullptr;
+        if (n < 16384) return nullptr;
         if (c->wts)
             return variant_by_name(n >= kBoxGuardMinN ? "f32x2wbguard.sfold64.sym8k256"
-                                                      : "f32x2wguard.fold64.sym4k128");
+                                   : n >= 32768       ? "f32x2wguard.fold64.sym4k128"
+                                                      : "f32x2wguard.fold64.sym4k64");
         if (kahan)
             return variant_by_name(n >= kBoxGuardWideN ? "f32x2bguard.kahan.sym8k256"
                                    : n >= 36864        ? "f32x2guard.kahan.sym8k128"
-                                                       : "f32x2guard.kahan.sym4k128");
+                                   : n >= 32768        ? "f32x2guard.kahan.sym4k128"
+                                                       : "f32x2guard.kahan.sym4k64");
         return variant_by_name(n >= kBoxGuardWideN  ? "f32x2bguard.sfold64.sym8k256"
                                : n >= kBoxGuardMinN ? "f32x2bguard.sfold64.sym8k128"
-                               : n >= 36864         ? "f32x2guard.fold64.sym8k128"
-                                                    : "f32x2guard.fold64.sym4k128");
+                                                    : "f32x2guard.fold64.sym4k64");
     }
-    if (n < (c->wts ? 15360 : 14336)) return nullptr;
+    if (n < (c->wts || kahan ? 15361 : 14336)) return nullptr;
     if (c->wts)
-        return variant_by_name(n >= 28672 ? "f32x2w.fold64.sym8k256" : "f32x2w.fold64.sym4k128");
+        return variant_by_name(n >= 32768 ? "f32x2w.fold64.sym8k256" : "f32x2w.fold64.sym4k64");
     if (kahan)
-        return variant_by_name(n >= 28672 ? "f32x2.kahan.sym8k256" : "f32x2.kahan.sym4k128");
+        return variant_by_name(n >= 32768   ? "f32x2.kahan.sym8k256"
+                               : n >= 28672 ? "f32x2.kahan.sym8k64"
+                                            : "f32x2.kahan.sym4k64");
     return variant_by_name(n >= 196608  ? "f32x2.fold64.sym8k512"
-                           : n >= 28672 ? "f32x2.fold64.sym8k256"
-                                        : "f32x2.fold64.sym4k128");
+                           : n >= 49152 ? "f32x2.fold64.sym8k256"
+                           : n >= 32768 ? "f32x2.fold64.sym8k64"
+                                        : "f32x2.fold64.sym4k64");
 }
 
 const Variant *one_sided_variant(const pp_ctx *c);

@@ -40,13 +40,15 @@ std::vector<Variant> sym_variants()
 {
     return {
 #define S(nm, ...) make_sym<__VA_ARGS__>(nm)
-        S("f32x2.fold64.sym4k128", 4, 128, POS_SINGLE, false, false, 3),
+        S("f32x2.fold64.sym4k64", 4, 64, POS_SINGLE, false, false, 3),
+        S("f32x2.fold64.sym8k64", 8, 64, POS_SINGLE, false, false, 3),
         S("f32x2.fold64.sym8k256", 8, 256, POS_SINGLE, false, false, 3),
         S("f32x2.fold64.sym8k512", 8, 512, POS_SINGLE, false, false, 3),
-        S("f32x2.kahan.sym4k128", 4, 128, POS_SINGLE, false, true, 4),
+        S("f32x2.kahan.sym4k64", 4, 64, POS_SINGLE, false, true, 4),
+        S("f32x2.kahan.sym8k64", 8, 64, POS_SINGLE, false, true, 3),
         S("f32x2.kahan.sym8k256", 8, 256, POS_SINGLE, false, true, 3),
-        S("f32x2guard.fold64.sym4k128", 4, 128, POS_GUARDED, false, false, 4),
-        S("f32x2guard.fold64.sym8k128", 8, 128, POS_GUARDED, false, false, 3),
+        S("f32x2guard.fold64.sym4k64", 4, 64, POS_GUARDED, false, false, 4),
+        S("f32x2guard.kahan.sym4k64", 4, 64, POS_GUARDED, false, true, 4),
         S("f32x2guard.kahan.sym4k128", 4, 128, POS_GUARDED, false, true, 4),
         S("f32x2guard.kahan.sym8k128", 8, 128, POS_GUARDED, false, true, 3),
         S("f32x2bguard.sfold64.sym8k128", 8, 128, POS_GUARDED, false, false, 3, true),
@@ -54,8 +56,9 @@ std::vector<Variant> sym_variants()
         S("f32x2bguard.kahan.sym8k256", 8, 256, POS_GUARDED, false, true, 3, true),
         S("f32x2split.fold64.sym4k128", 4, 128, POS_SPLIT, false, false, 4),
         S("f32x2split.kahan.sym4k128", 4, 128, POS_SPLIT, false, true, 4),
-        S("f32x2w.fold64.sym4k128", 4, 128, POS_SINGLE, true, false, 4),
+        S("f32x2w.fold64.sym4k64", 4, 64, POS_SINGLE, true, false, 4),
         S("f32x2w.fold64.sym8k256", 8, 256, POS_SINGLE, true, false, 2),
+        S("f32x2wguard.fold64.sym4k64", 4, 64, POS_GUARDED, true, false, 4),
         S("f32x2wguard.fold64.sym4k128", 4, 128, POS_GUARDED, true, false, 4),
         S("f32x2wbguard.sfold64.sym8k256", 8, 256, POS_GUARDED, true, false, 2, true),
         S("f32x2wsplit.fold64.sym4k128", 4, 128, POS_SPLIT, true, false, 3),
