@@ -9,9 +9,9 @@
 // two targets per lane in registers, the sources of a block broadcast from its
 // shared memory.  Per pair: 7 f32x2 half-instructions and one SFU rsqrt, which
 // bounds the loop (one operation per pair at 16 per clock and SM).  FP32 sums of
-// 256 terms fold into FP64.  N = 100003: 1.20 ms, 83 % of that bound (the
-// one-sided scalar loop with its index and zero tests took 4.0); N = 2048: 26 us
-// against 73.
+// 64, 128 (from N = 16384) or 256 terms (from 32768, where 128 cost 2 %) fold into
+// FP64.  N = 100003: 1.19 ms, 84 % of that bound (the one-sided scalar loop with its
+// index and zero tests took 4.0); N = 24001: 94 us; N = 2048: 25 us against 73.
 #include "pp_internal.h"
 
 namespace ppk {
@@ -20,18 +20,18 @@ namespace {
 
 constexpr int kWarps = 4;
 
-// FP32 sums of w_j / sqrt(s) of each target over the sources of `tile`.  MASKED:
-// zero-distance pairs are left out, and with `self` >= 0 the pair of a target
-// with itself (self: the lane).
-template <int PK, bool MASKED>
-__device__ __forceinline__ void block_terms(const float4 *tile, const f2_t (&X)[PK],
+// FP32 sums of w_j / sqrt(s) of each target over the LEN sources from `first` on of
+// `tile`.  MASKED: zero-distance pairs are left out, and with `self` >= 0 the pair of a
+// target with itself (self: the lane).
+template <int PK, int LEN, bool MASKED>
+__device__ __forceinline__ void block_terms(const float4 *tile, int first, const f2_t (&X)[PK],
                                             const f2_t (&Y)[PK], const f2_t (&Z)[PK], f2_t EPS2,
                                             int self, f2_t (&F)[PK])
 {
 #pragma unroll
     for (int k = 0; k < PK; ++k) F[k] = 0ull;
 #pragma unroll 4
-    for (int j = 0; j < 64 * PK; ++j) {
+    for (int j = first; j < first + LEN; ++j) {
         const float4 s = tile[j];   // padding sources carry s.w = 0
         const f2_t XJ = f2_pack(s.x, s.x), YJ = f2_pack(s.y, s.y), ZJ = f2_pack(s.z, s.z);
         const f2_t WJ = f2_pack(s.w, s.w);
@@ -52,12 +52,14 @@ __device__ __forceinline__ void block_terms(const float4 *tile, const f2_t (&X)[
     }
 }
 
-template <int PK>
+// LEN: terms per FP32 sum.
+template <int PK, int LEN>
 __global__ void __launch_bounds__(32 * kWarps, 4)
     potential_kernel(const float4 *__restrict__ src, int n, int nb, int nd, int chunk, float eps2,
                      const double *__restrict__ wts, double *partials, int count)
 {
     constexpr int B = 64 * PK;   // particles per block
+    static_assert(B % LEN == 0, "whole sums per block");
     __shared__ float4 sm[kWarps][B];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int id = blockIdx.x * kWarps + warp;   // this warp's (block, range) and result slot
@@ -84,24 +86,28 @@ __global__ void __launch_bounds__(32 * kWarps, 4)
         __syncwarp();
         for (int e = lane; e < B; e += 32) tile[e] = src[jb * B + e];
         __syncwarp();
-        bool again = d == 0;
-        if (!again) {
-            block_terms<PK, false>(tile, X, Y, Z, EPS2, -1, F);
-            f2_t all = F[0];
-#pragma unroll
-            for (int k = 1; k < PK; ++k) all = f2_add(all, F[k]);
-            float a, b;
-            f2_unpack(all, a, b);
-            again = __any_sync(0xffffffffu, !isfinite(a + b));   // a zero-distance pair
-        }
-        if (again) block_terms<PK, true>(tile, X, Y, Z, EPS2, d == 0 ? lane : -1, F);
         const double share = d == 0 ? 0.5 : 1.0;
+#pragma unroll 1
+        for (int first = 0; first < B; first += LEN) {
+            bool again = d == 0;
+            if (!again) {
+                block_terms<PK, LEN, false>(tile, first, X, Y, Z, EPS2, -1, F);
+                f2_t all = F[0];
 #pragma unroll
-        for (int k = 0; k < PK; ++k) {
-            float a, b;
-            f2_unpack(F[k], a, b);
-            acc[2 * k] += share * (double)a;
-            acc[2 * k + 1] += share * (double)b;
+                for (int k = 1; k < PK; ++k) all = f2_add(all, F[k]);
+                float a, b;
+                f2_unpack(all, a, b);
+                again = __any_sync(0xffffffffu, !isfinite(a + b));   // a zero-distance pair
+            }
+            if (again)
+                block_terms<PK, LEN, true>(tile, first, X, Y, Z, EPS2, d == 0 ? lane : -1, F);
+#pragma unroll
+            for (int k = 0; k < PK; ++k) {
+                float a, b;
+                f2_unpack(F[k], a, b);
+                acc[2 * k] += share * (double)a;
+                acc[2 * k + 1] += share * (double)b;
+            }
         }
     }
     double sum = 0.0;
@@ -131,7 +137,7 @@ __global__ void __launch_bounds__(1024) potential_sum_kernel(const double *parti
     }
 }
 
-template <int PK>
+template <int PK, int LEN>
 int run_potential(const void *src, int n, float eps2, const double *wts, double *partials,
                   cudaStream_t s)
 {
@@ -142,7 +148,7 @@ int run_potential(const void *src, int n, float eps2, const double *wts, double 
     ranges = ranges < 1 ? 1 : ranges > 16 * PK ? 16 * PK : ranges;
     const int chunk = (nd + ranges - 1) / ranges;
     const int count = nb * ((nd + chunk - 1) / chunk);
-    potential_kernel<PK><<<(count + kWarps - 1) / kWarps, 32 * kWarps, 0, s>>>(
+    potential_kernel<PK, LEN><<<(count + kWarps - 1) / kWarps, 32 * kWarps, 0, s>>>(
         static_cast<const float4 *>(src), n, nb, nd, chunk, eps2, wts, partials, count);
     return count;
 }
@@ -154,8 +160,9 @@ cudaError_t launch_potential(const void *src, int n, int npad, float eps2, const
                              double *partials, double *out, cudaStream_t s)
 {
     if (n < 1 || npad < n || npad % 256 != 0) return cudaErrorInvalidValue;
-    const int count = n < 16384 ? run_potential<1>(src, n, eps2, wts, partials, s)
-                                : run_potential<4>(src, n, eps2, wts, partials, s);
+    const int count = n < 16384   ? run_potential<1, 64>(src, n, eps2, wts, partials, s)
+                      : n < 32768 ? run_potential<4, 128>(src, n, eps2, wts, partials, s)
+                                  : run_potential<4, 256>(src, n, eps2, wts, partials, s);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     potential_sum_kernel<<<1, 1024, 0, s>>>(partials, count, out);

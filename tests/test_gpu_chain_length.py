@@ -58,3 +58,28 @@ def test_fields_add_at_most_64_terms_in_fp32(n, acc, mode, weighted):
     err = np.linalg.norm(E[idx] - ref, axis=1) / np.linalg.norm(ref, axis=1)
     rms = float(np.sqrt(np.mean(err ** 2)))
     assert rms <= LIMIT, f"rms error {rms / U32:.1f} u"
+
+
+def two_clusters(n, gap):
+    pos = np.zeros((n, 3))
+    pos[n // 2:] = gap * np.array([0.48, 0.6, 0.64])
+    return pos
+
+
+@pytest.mark.parametrize("n", [16384, 24001, 32767])
+def test_potential_energy_adds_at_most_128_terms_in_fp32(n):
+    """Two clusters of coincident particles: the potential energy is n_A n_B equal terms (the
+    zero-distance pairs add nothing).  The limit lies half way between chains of 128 and 256."""
+    limit = float(np.sqrt(chain_rms(128) * chain_rms(256)))
+    c = oracle.constants()
+    err = []
+    with capi.Simulation(n, 12.0, 1e-16, 0.0, positions=SINGLE) as sim:
+        for gap in 1e-5 * (0.5 + 1.5 * wl.uniform(19, 1, 32)):
+            pos = two_clusters(n, gap)
+            sim.load(pos)
+            got = sim.diagnostics()["pe"]
+            pairs = float(n // 2) * (n - n // 2)
+            want = c["k"] * c["e"] ** 2 * 12.0 ** 2 * pairs / np.linalg.norm(pos[-1])
+            err.append((got - want) / want)
+    rms = float(np.sqrt(np.mean(np.square(err))))
+    assert rms <= limit, f"rms error {rms / U32:.1f} u of {limit / U32:.1f}"
