@@ -182,13 +182,16 @@ typedef enum {
  * Create a context for N macro-electrons of common weight w (Sec. 2.1 assumes
  * one weight for all macro-particles), time step dt > 0 and softening
  * eps >= 0 (metres).  Allocates the state and staging buffers on the current
- * CUDA device; force passes allocate their workspaces on first use (the partial
- * sums, 1 to 5 KB per particle where the pair-symmetric kernels run, which is by
- * default from about N = 15000 to 2^22; with guarded staging from N = 98304 on,
- * the spatial-order workspace, 44 to 52 bytes per particle) and return
- * PP_ERR_NOMEM if that fails; without room for the partial sums of the symmetric
- * kernels a context goes on with the one-sided ones.  N >= 1 (N = 0 -> PP_ERR_ARG); N <= 2^28.  On success *out receives
- * the context; on failure *out is set to NULL.
+ * CUDA device; force passes allocate their workspaces on first use (with guarded
+ * staging from N = 98304 on, the spatial-order workspace, 44 to 52 bytes per
+ * particle) and return PP_ERR_NOMEM if that fails.  The pair-symmetric kernels,
+ * by default from about N = 15000 to 2^22 (all-FP64: from 1), keep partial sums of
+ * 1 to 7 KB per particle (6 GB at 2^20).  They take at most a quarter of the
+ * device memory that is free at that moment; without that much a context goes on
+ * with the one-sided kernels, which need none, until an option that picks the
+ * kernel is set or particles are loaded.  Setting PP_OPT_SPLIT to another value
+ * gives them back.  N >= 1 (N = 0 -> PP_ERR_ARG); N <= 2^28.  On success *out
+ * receives the context; on failure *out is set to NULL.
  */
 pp_status pp_create(int64_t N, double w, double dt, double softening, pp_ctx **out);
 

@@ -86,7 +86,9 @@ struct pp_ctx {
     std::vector<SymEntry> sym;
     double *sym_ws = nullptr;
     size_t sym_ws_bytes = 0;
-    bool sym_off = false;          // the partial sums could not be allocated
+    bool sym_off = false;          // no room for the partial sums (until an option or a load)
+    bool sym_whole = false;        // no room for those of the split asked for: its own ranges
+    bool tuning = false;           // pp_autotune sets the variant, not the caller
     double *mom_host = nullptr;    // pinned
     int *err_host = nullptr;       // pinned copy of err[0..1], read after each synchronisation
 
@@ -172,14 +174,14 @@ constexpr int64_t kBoxGuardWideN = 196608;
 // 8 % at N = 32768, single (0.341 against 0.314 with 256), 0 to 5 % with the blocks of
 // 256 targets.  Those blocks are faster below N = 32768 (Kahan, 28672) and, with the test
 // per pair, at every N (guarded 65536: 1.26 against 1.30 with 512).  Above 2^22 the
-// partial sums would pass 18 GB for a step of seconds: one-sided again.
+// partial sums would pass 29 GB for a step of seconds: one-sided again.
 constexpr int64_t kSymMaxN = int64_t(1) << 22;
 const Variant *sym_variant(const pp_ctx *c)
 {
     const int64_t n = c->n;
     const bool kahan = c->acc == PP_ACC_KAHAN;
     if (c->sym_off || n > kSymMaxN) return nullptr;
-    if (f64_pairs(c))   // faster at every N (0.058 / 0.174 ms at N = 1000, 5.03 / 10.4 at 16385)
+    if (f64_pairs(c))   // faster at every N (0.058 / 0.174 ms at N = 1000, 5.1 / 10.4 at 16385)
         return variant_by_name(c->wts ? "f64w.full.symr1k32" : "f64.full.symr1k32");
     if (c->positions == PP_POS_SPLIT) {
         if (n < 13000) return nullptr;
@@ -357,6 +359,7 @@ int resident_ctas(const Variant &v)
 struct Plan {
     const Variant *v;
     int nib, nsplit, jchunk, grid, nipad;
+    int sym_at;   // symmetric: the plan's place in c->sym (ensure_workspace)
 };
 
 // Choose S, the number of j-chunks per i-block, to fill the GPU: minimise
@@ -414,11 +417,12 @@ Plan make_plan(pp_ctx *c, int kind)
 constexpr size_t kSymPlans = 8;
 
 // Device tables and partial sums of a pair-symmetric pass, made once per
-// (variant, split) of the context.  *at: its place in c->sym.
-pp_status ensure_sym(pp_ctx *c, const Variant &v, int *at)
+// (variant, split) of the context.  *at: its place in c->sym.  The sums take at most a
+// quarter of the free memory (sym_sums_fit) unless the caller named the variant.
+pp_status ensure_sym(pp_ctx *c, const Variant &v, int split, int *at)
 {
     int count = 0;
-    const std::pair<int, int> key{(int)(&v - variants(&count)), c->split_override};
+    const std::pair<int, int> key{(int)(&v - variants(&count)), split};
     for (size_t k = 0; k < c->sym.size(); ++k)
         if (c->sym[k].key == key) {
             *at = (int)k;
@@ -426,10 +430,16 @@ pp_status ensure_sym(pp_ctx *c, const Variant &v, int *at)
         }
     const int64_t slots = (int64_t)c->sms * resident_ctas(v);
     const SymPlan sp = make_sym_plan((int)c->n, c->npad, 32 * v.R, v.kind == KIND_FORCE64, slots,
-                                     c->split_override);
+                                     split);
     const size_t ib = round_up(sp.items.size() * sizeof(SymItem), 256);
     const size_t rb = round_up(sp.rows.size() * sizeof(SymRow), 256);
     const size_t ws = (sp.row_doubles + sp.part_doubles) * sizeof(double);
+    if (ws > c->sym_ws_bytes && (c->variant_override < 0 || c->tuning)) {
+        size_t free = 0, total = 0;
+        PP_CUDA(cudaMemGetInfo(&free, &total));
+        if (!sym_sums_fit(ws, free + c->sym_ws_bytes))
+            return fail(PP_ERR_NOMEM, "the symmetric pass would take too much of the free memory");
+    }
     // a pass with the old buffers may be running, or captured in a graph
     if (ws > c->sym_ws_bytes || c->sym.size() >= kSymPlans) {
         drop_graphs(c);
@@ -482,11 +492,17 @@ pp_status ensure_sym(pp_ctx *c, const Variant &v, int *at)
     return PP_OK;
 }
 
-pp_status ensure_workspace(pp_ctx *c, const Plan &pl)
+pp_status ensure_workspace(pp_ctx *c, Plan &pl)
 {
-    int at = 0;
-    if (pl.v->sym)
-        if (pp_status st = ensure_sym(c, *pl.v, &at)) return st;
+    if (pl.v->sym) {
+        const int split = c->sym_whole ? 0 : c->split_override;
+        pp_status st = ensure_sym(c, *pl.v, split, &pl.sym_at);
+        if (st == PP_ERR_NOMEM && split > 0) {   // fine ranges need many more sums
+            c->sym_whole = true;
+            st = ensure_sym(c, *pl.v, 0, &pl.sym_at);
+        }
+        if (st != PP_OK) return st;
+    }
     if (pl.v->order) {
         const size_t need = order_workspace_bytes(c->npad, pl.v->tile);
         if (need > c->ord_bytes) {
@@ -604,19 +620,18 @@ cudaError_t launch_force(pp_ctx *c, const Plan &pl, ForceArgs a)
         a.boxes = w.boxes;
     }
     if (pl.v->sym) {
-        int at = 0;
-        if (ensure_sym(c, *pl.v, &at) != PP_OK) return cudaErrorMemoryAllocation;   // made already
-        SymArgs q = c->sym[at].args;
+        const pp_ctx::SymEntry &e = c->sym[pl.sym_at];
+        SymArgs q = e.args;
         q.jrow = c->sym_ws;
-        q.ipart = c->sym_ws + c->sym[at].row_doubles;
-        return launch_sym(*pl.v, a, q, c->sym[at].grid, c->stream);
+        q.ipart = c->sym_ws + e.row_doubles;
+        return launch_sym(*pl.v, a, q, e.grid, c->stream);
     }
     return launch_variant(*pl.v, a, pl.grid, c->stream);
 }
 
 // The plan of a pass with its workspaces.  Where the default plan is symmetric
-// and its partial sums cannot be allocated, the context goes on with the
-// one-sided kernels.
+// and there is no room for its partial sums, the context goes on with the
+// one-sided kernels until an option is set or particles are loaded (retry_sym).
 pp_status plan_pass(pp_ctx *c, int kind, Plan *pl)
 {
     *pl = make_plan(c, kind);
@@ -628,6 +643,24 @@ pp_status plan_pass(pp_ctx *c, int kind, Plan *pl)
         st = ensure_workspace(c, *pl);
     }
     return st;
+}
+
+// Memory may have been given back, or the plan may need less now.
+void retry_sym(pp_ctx *c)
+{
+    if (c->sym_off || c->sym_whole) drop_graphs(c);
+    c->sym_off = c->sym_whole = false;
+}
+
+// Give the partial sums and the plans back (no pass runs).
+void drop_sym(pp_ctx *c)
+{
+    drop_graphs(c);
+    for (auto &e : c->sym) cudaFree(e.tab);
+    c->sym.clear();
+    cudaFree(c->sym_ws);
+    c->sym_ws = nullptr;
+    c->sym_ws_bytes = 0;
 }
 
 // One force pass over staged sources src.
@@ -1123,8 +1156,7 @@ pp_status pp_destroy(pp_ctx *c)
     cudaFree(c->err);
     cudaFree(c->res_flags);
     cudaFree(c->ord_ws);
-    for (auto &e : c->sym) cudaFree(e.tab);
-    cudaFree(c->sym_ws);
+    drop_sym(c);
     if (c->mom_host) cudaFreeHost(c->mom_host);
     if (c->err_host) cudaFreeHost(c->err_host);
     if (c->own_stream) cudaStreamDestroy(c->own_stream);
@@ -1196,6 +1228,8 @@ pp_status pp_create(int64_t N, double w, double dt, double softening, pp_ctx **o
 pp_status pp_set_option(pp_ctx *c, int key, int64_t value)
 {
     if (pp_status s = check_ctx(c)) return s;
+    if (key == PP_OPT_ACC || key == PP_OPT_POSITIONS || key == PP_OPT_SPLIT || key == PP_OPT_VARIANT)
+        retry_sym(c);
     switch (key) {
     case PP_OPT_ACC:
     case PP_OPT_POSITIONS: {
@@ -1228,6 +1262,10 @@ pp_status pp_set_option(pp_ctx *c, int key, int64_t value)
         return PP_OK;
     case PP_OPT_SPLIT:
         if (value < 0 || value > 4096) return fail(PP_ERR_ARG, "split must be in [0, 4096]");
+        if (c->split_override != (int)value && !c->sym.empty()) {
+            PP_CUDA(cudaSetDevice(c->device));
+            drop_sym(c);   // a fine split's sums can be ten times the automatic plan's
+        }
         c->split_override = (int)value;
         drop_graphs(c);
         return PP_OK;
@@ -1306,6 +1344,7 @@ pp_status pp_load_particles(pp_ctx *c, const double *pos, const double *vel, int
     if (!valid_mem(on_device)) return fail(PP_ERR_ARG, "bad memory kind");
     PP_CUDA(cudaSetDevice(c->device));
     drop_graphs(c);
+    retry_sym(c);
     c->loaded = false;
     pp_status st = import_aos(c, pos, on_device, c->r);
     if (st != PP_OK) return st;
@@ -1620,6 +1659,11 @@ pp_status pp_autotune(pp_ctx *c, pp_tune_result *out)
     int count = 0;
     const Variant *vs = variants(&count);
     const int saved_variant = c->variant_override, saved_split = c->split_override;
+    struct Tuning {   // candidates take memory by the rule of a default plan
+        pp_ctx *c;
+        explicit Tuning(pp_ctx *ctx) : c(ctx) { c->tuning = true; }
+        ~Tuning() { c->tuning = false; }
+    } tuning_(c);
     const int old_kind = stage_kind(c);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     PP_CUDA(cudaEventCreate(&e0));

@@ -47,6 +47,11 @@ struct SymPlan {
     size_t row_doubles = 0, part_doubles = 0;
 };
 
+// May a pass take `bytes` for its partial sums with `free` bytes left on the device?
+// A quarter of them at most: what else shares the GPU (other contexts, the program's
+// own arrays) still finds room, and the pass has a one-sided form that needs none.
+inline bool sym_sums_fit(size_t bytes, size_t free) { return bytes <= free / 4; }
+
 // Work items of one pass over blocks of `targets` particles with `slots` CTAs
 // resident: each group of ki target blocks walks the sources from its own start to
 // the end; its row is cut into ranges of half a resident warp's share of the
@@ -65,8 +70,8 @@ struct SymPlan {
 // split > 0 shortens the ranges to npad / split where they are longer; it never
 // lengthens them, since the warps without work wait for the last item, and a row
 // on one warp takes seconds at N = 2^20.  Each item keeps its own sums, which
-// bounds how finely the work may be cut: rows and items take 5 KB per particle at
-// 2^20.
+// bounds how finely the work may be cut: rows and items take 4 to 7 KB per particle
+// from N = 65536 on.
 inline SymPlan make_sym_plan(int n, int npad, int targets, bool f64, int64_t slots, int split)
 {
     SymPlan pl;

@@ -119,3 +119,27 @@ def test_the_last_round_of_items_is_not_nearly_empty(driver, n, targets, slots):
     of N = 13001 (1.77).  A third over the even share is what one whole round of two to four
     costs at worst; the warps of a scheduler speed up when one of them has run out of work."""
     assert driver([(n, targets, 0, slots, 0)])[0][4] <= 4.0 / 3.0
+
+
+FITS = r"""
+#include <cstdio>
+#include "pp_sym_plan.h"
+int main()
+{
+    using ppk::sym_sums_fit;
+    const size_t gb = size_t(1) << 30;
+    printf("%d%d%d%d%d", sym_sums_fit(0, 0), sym_sums_fit(1, 3), sym_sums_fit(6 * gb, 24 * gb),
+           sym_sums_fit(6 * gb + 1, 24 * gb), sym_sums_fit(29 * gb, 270 * gb));
+}
+"""
+
+
+def test_partial_sums_take_a_quarter_of_the_free_memory_at_most(tmp_path):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if cxx is None:
+        pytest.skip("no C++ compiler")
+    (tmp_path / "fits.cpp").write_text(FITS)
+    exe = str(tmp_path / "fits")
+    subprocess.run([cxx, "-std=c++17", "-I", build.CSRC, str(tmp_path / "fits.cpp"), "-o", exe],
+                   check=True)
+    assert subprocess.run([exe], check=True, capture_output=True, text=True).stdout == "10101"
