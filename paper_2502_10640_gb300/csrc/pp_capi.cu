@@ -294,12 +294,6 @@ const Variant *one_sided_variant(const pp_ctx *c)
 // Staging layout the force kernels of this context read.
 int stage_kind(const pp_ctx *c) { return force_variant(c)->stage; }
 
-// Pick the variant for a kind of pass.
-const Variant *pick_variant(const pp_ctx *c, int kind)
-{
-    return force_variant(c);
-}
-
 // Can at least one cluster of this variant be resident on the device?
 bool cluster_fits(const Variant &v)
 {
@@ -364,10 +358,10 @@ struct Plan {
 
 // Choose S, the number of j-chunks per i-block, to fill the GPU: minimise
 // (waves of CTAs) x (tiles per CTA + fixed per-CTA overhead).
-Plan make_plan(pp_ctx *c, int kind)
+Plan make_plan(const pp_ctx *c)
 {
     Plan pl{};
-    pl.v = pick_variant(c, kind);
+    pl.v = force_variant(c);
     const int BI = pl.v->T * pl.v->R;
     pl.nib = (int)((c->n + BI - 1) / BI);
     pl.nipad = pl.nib * BI;
@@ -632,14 +626,14 @@ cudaError_t launch_force(pp_ctx *c, const Plan &pl, ForceArgs a)
 // The plan of a pass with its workspaces.  Where the default plan is symmetric
 // and there is no room for its partial sums, the context goes on with the
 // one-sided kernels until an option is set or particles are loaded (retry_sym).
-pp_status plan_pass(pp_ctx *c, int kind, Plan *pl)
+pp_status plan_pass(pp_ctx *c, Plan *pl)
 {
-    *pl = make_plan(c, kind);
+    *pl = make_plan(c);
     pp_status st = ensure_workspace(c, *pl);
     if (st == PP_ERR_NOMEM && pl->v->sym && pl->v == sym_variant(c)) {
         c->sym_off = true;
         drop_graphs(c);
-        *pl = make_plan(c, kind);
+        *pl = make_plan(c);
         st = ensure_workspace(c, *pl);
     }
     return st;
@@ -666,9 +660,8 @@ void drop_sym(pp_ctx *c)
 // One force pass over staged sources src.
 pp_status force_pass(pp_ctx *c, int mode, const void *src, void *dst, double *out)
 {
-    const int kind = f64_pairs(c) ? KIND_FORCE64 : KIND_FORCE32;
     Plan pl{};
-    pp_status st = plan_pass(c, kind, &pl);
+    pp_status st = plan_pass(c, &pl);
     if (st != PP_OK) return st;
     ForceArgs a = base_args(c, pl, mode, src, dst, out);
     a.skip_copy = c->skip_copy;
@@ -870,9 +863,8 @@ bool graph_capturable(const pp_ctx *c) { return c->graph_block > 0 && c->stream 
 pp_status build_graphs(pp_ctx *c)
 {
     drop_graphs(c);
-    const int kind = f64_pairs(c) ? KIND_FORCE64 : KIND_FORCE32;
     Plan pl{};
-    pp_status st = plan_pass(c, kind, &pl);
+    pp_status st = plan_pass(c, &pl);
     if (st != PP_OK) return st;
     for (int p0 = 0; p0 < 2; ++p0) {
         cudaGraph_t g = nullptr;
@@ -1687,7 +1679,7 @@ pp_status pp_autotune(pp_ctx *c, pp_tune_result *out)
         if (vs[v].sym && (c->sym_off || c->n > kSymMaxN)) continue;   // partial sums too large
         c->variant_override = v;
         c->split_override = 0;
-        const Plan base = make_plan(c, vs[v].kind);
+        const Plan base = make_plan(c);
         const int tiles = c->npad / vs[v].tile;
         int cand[4] = {base.nsplit, std::max(1, base.nsplit / 2), std::min(tiles, 2 * base.nsplit),
                        std::max(1, base.nsplit / 4)};

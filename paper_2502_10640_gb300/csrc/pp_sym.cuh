@@ -339,8 +339,7 @@ __device__ __forceinline__ void sym_collect(const ForceArgs &p, const SymArgs &q
 // pair (non-finite sum) or, with POS_GUARDED, with a pair too close for the hi
 // parts alone.  BOX: the caller has ruled close pairs out.  Not inlined: the loop needs every register for
 // itself (inlined into the queue loop it ran 10 % slower).
-template <int PK, int TJ, int WI, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, bool ADD,
-          int MINB>
+template <int PK, int TJ, int WI, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, bool ADD>
 __device__ __noinline__ bool sym_tile(const float *__restrict__ src, size_t lo_at, int n, int i0,
                                       int j0, int count, float eps2, double *acc, int at0, float *stash)
 {
@@ -479,17 +478,17 @@ __device__ __noinline__ bool sym_tile(const float *__restrict__ src, size_t lo_a
 
 // A tile on hi/lo separations, four packs at a time (the lo parts take as many
 // registers as the hi parts).
-template <int PK, int TJ, int WI, bool WEIGHTED, bool KAHAN, bool OWN, int MINB>
+template <int PK, int TJ, int WI, bool WEIGHTED, bool KAHAN, bool OWN>
 __device__ __forceinline__ void sym_split(const float *src, size_t lo_at, int n, int i0, int j0,
                                           int count, float eps2, double *acc, float *stash)
 {
     constexpr int PH = PK > 4 ? 4 : PK;
     static_assert(PK == PH || PK == 2 * PH, "one or two parts");
-    if (!sym_tile<PH, TJ, WI, POS_SPLIT, false, WEIGHTED, KAHAN, OWN, false, MINB>(
+    if (!sym_tile<PH, TJ, WI, POS_SPLIT, false, WEIGHTED, KAHAN, OWN, false>(
             src, lo_at, n, i0, j0, count, eps2, acc, 0, stash))
         sym_slow<PH, TJ, WI, true, WEIGHTED, KAHAN, OWN>(src, lo_at, n, i0, j0, count, eps2, acc, 0, stash,
                                                         false, true);
-    if (PK > PH && !sym_tile<PH, TJ, WI, POS_SPLIT, false, WEIGHTED, KAHAN, OWN, true, MINB>(
+    if (PK > PH && !sym_tile<PH, TJ, WI, POS_SPLIT, false, WEIGHTED, KAHAN, OWN, true>(
                        src, lo_at, n, i0 + 64 * PH, j0, count, eps2, acc, 64 * PH, stash)) {
         // the first part's share of the source sums again, then this part
         if (!OWN)
@@ -502,17 +501,17 @@ __device__ __forceinline__ void sym_split(const float *src, size_t lo_at, int n,
 
 // One (warp, tile) by whichever of the forms above it needs.  close: BOX found
 // that it may hold close pairs.
-template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, int MINB>
+template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN>
 __device__ __forceinline__ void sym_any(const float *src, size_t lo_at, int n, int i0, int j0,
                                         int count, float eps2, double *acc, float *stash, bool close)
 {
     constexpr int WI = 64 * PK;
     if (!(BOX && close) &&
-        sym_tile<PK, TJ, WI, POS, BOX, WEIGHTED, KAHAN, OWN, false, MINB>(
+        sym_tile<PK, TJ, WI, POS, BOX, WEIGHTED, KAHAN, OWN, false>(
             src, lo_at, n, i0, j0, count, eps2, acc, 0, stash))
         return;
     if (POS == POS_GUARDED)
-        sym_split<PK, TJ, WI, WEIGHTED, KAHAN, OWN, MINB>(src, lo_at, n, i0, j0, count, eps2, acc, stash);
+        sym_split<PK, TJ, WI, WEIGHTED, KAHAN, OWN>(src, lo_at, n, i0, j0, count, eps2, acc, stash);
     else
         sym_slow<PK, TJ, WI, POS == POS_SPLIT, WEIGHTED, KAHAN, OWN>(src, lo_at, n, i0, j0, count, eps2,
                                                                     acc, 0, stash, false, true);
@@ -597,10 +596,10 @@ __global__ void __launch_bounds__(kSymThreads, MINB)
                 const bool mine = j < i0 + WI;   // the sources are among the targets
                 len = min(TJ - j % TJ, it.j1 - j);
                 if (mine)
-                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, true, MINB>(
+                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, true>(
                         src, lo_at, p.n, i0, j, len, p.eps2f, acc, stash, true);
                 else
-                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, false, MINB>(
+                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, false>(
                         src, lo_at, p.n, i0, j, len, p.eps2f, acc, stash,
                         BOX && __any_sync(0xffffffffu, sym_box_close(p.boxes, j / TJ, lo, hi, rmax2,
                                                                      p.eps2f)));
