@@ -446,7 +446,7 @@ const char *pp_last_error(const pp_ctx *ctx);
  * "f32x2.fold64.t256r4k256": packed FP32x2 pair math, FP64 fold, 256 threads,
  * 4 targets per thread, 256-source tiles; or "<pairs>.<fold>.sym<packs>k<tile>"
  * for the pair-symmetric kernels (each unordered pair evaluated once), `packs`
- * pairs of targets per thread.
+ * pairs of targets per thread (h: the two halves of a tile summed apart).
  */
 const char *pp_variant_name(int index);
 

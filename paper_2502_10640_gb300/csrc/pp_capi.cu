@@ -158,7 +158,7 @@ constexpr int64_t kBoxGuardWideN = 196608;
 // small N leaves too few units; from there on it runs 14 FP32 lane operations per
 // unordered pair instead of 22.  The lines lie where the GB300 sweep has the two
 // level.  ms per step, symmetric / one-sided:
-//   single         0.090 / 0.101 at N = 14336, 0.206 / 0.241 at 24001, 0.341 / 0.407 at
+//   single         0.090 / 0.101 at N = 14336, 0.206 / 0.241 at 24001, 0.320 / 0.407 at
 //                  32768, 1.12 / 1.47 at 65536, 4.37 / 5.79 at 131072, 16.8 / 22.5 at 262144
 //   Kahan          0.106 / 0.099 at 14336, 0.114 / 0.117 at 15361, 0.319 / 0.452 at 32768
 //   weights        0.110 / 0.109 at 14336, 0.128 / 0.128 at 15361, 0.130 / 0.139 at 16385,
@@ -170,10 +170,10 @@ constexpr int64_t kBoxGuardWideN = 196608;
 //                  Kahan 0.114 / 0.163 at 13001, weights 0.108 / 0.166
 // The tiles (64 to 512 sources) keep the FP32 partial sum of a target no longer than
 // that of the one-sided kernel that would run instead: 64 terms below N = 49152 (Kahan
-// and weights 32768, guarded 98304), 128 to 512 above.  Folding every 64 sources costs
-// 8 % at N = 32768, single (0.341 against 0.314 with 256), 0 to 5 % with the blocks of
-// 256 targets.  Those blocks are faster below N = 32768 (Kahan, 28672) and, with the test
-// per pair, at every N (guarded 65536: 1.26 against 1.30 with 512).  Above 2^22 the
+// and weights 32768, guarded 98304), 128 to 512 above.  That costs 2 % at N = 32768,
+// single (0.320 against 0.314 with 256 terms), 0 to 5 % with the blocks of 256 targets.
+// Those blocks are faster below N = 28672 (weights, 32768) and, with the test per pair,
+// at every N (guarded 65536: 1.26 against 1.30 with 512).  Above 2^22 the
 // partial sums would pass 29 GB for a step of seconds: one-sided again.
 constexpr int64_t kSymMaxN = int64_t(1) << 22;
 const Variant *sym_variant(const pp_ctx *c)
@@ -213,7 +213,7 @@ const Variant *sym_variant(const pp_ctx *c)
                                             : "f32x2.kahan.sym4k64");
     return variant_by_name(n >= 196608  ? "f32x2.fold64.sym8k512"
                            : n >= 49152 ? "f32x2.fold64.sym8k256"
-                           : n >= 32768 ? "f32x2.fold64.sym8k64"
+                           : n >= 28672 ? "f32x2.fold64.sym8k128h"
                                         : "f32x2.fold64.sym4k64");
 }
 

@@ -7,13 +7,14 @@ namespace ppk {
 
 namespace {
 
-template <int PK, int TJ, int POS, bool WEIGHTED, bool KAHAN, int MINB, bool BOX = false>
+template <int PK, int TJ, int POS, bool WEIGHTED, bool KAHAN, int MINB, bool BOX = false,
+          bool HALF = false>
 Variant make_sym(const char *name)
 {
     Variant v{name, WEIGHTED ? KIND_FORCE32W : KIND_FORCE32, KAHAN ? ACC_KAHAN : ACC_FP64FOLD,
               POS == POS_SINGLE ? STAGE_F32I : STAGE_F32IX2, kSymThreads, 2 * PK, TJ, 0,
               reinterpret_cast<const void *>(
-                  &force_sym_kernel<PK, TJ, POS, BOX, WEIGHTED, KAHAN, MINB>),
+                  &force_sym_kernel<PK, TJ, POS, BOX, WEIGHTED, KAHAN, MINB, HALF>),
               kSymWarps * sym_warp_smem<PK, TJ>(), 0, POS, BOX ? 1 : 0};
     v.sym = 1;
     return v;
@@ -41,7 +42,7 @@ std::vector<Variant> sym_variants()
     return {
 #define S(nm, ...) make_sym<__VA_ARGS__>(nm)
         S("f32x2.fold64.sym4k64", 4, 64, POS_SINGLE, false, false, 3),
-        S("f32x2.fold64.sym8k64", 8, 64, POS_SINGLE, false, false, 3),
+        S("f32x2.fold64.sym8k128h", 8, 128, POS_SINGLE, false, false, 3, false, true),
         S("f32x2.fold64.sym8k256", 8, 256, POS_SINGLE, false, false, 3),
         S("f32x2.fold64.sym8k512", 8, 512, POS_SINGLE, false, false, 3),
         S("f32x2.kahan.sym4k64", 4, 64, POS_SINGLE, false, true, 4),

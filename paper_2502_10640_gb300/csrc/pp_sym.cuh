@@ -337,9 +337,13 @@ __device__ __forceinline__ void sym_collect(const ForceArgs &p, const SymArgs &q
 // only (the pair comes again with the roles exchanged) and skips itself by index.  Returns false (for
 // the whole warp, nothing folded, stash void) for a tile with a zero-distance
 // pair (non-finite sum) or, with POS_GUARDED, with a pair too close for the hi
-// parts alone.  BOX: the caller has ruled close pairs out.  Not inlined: the loop needs every register for
-// itself (inlined into the queue loop it ran 10 % slower).
-template <int PK, int TJ, int WI, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, bool ADD>
+// parts alone.  BOX: the caller has ruled close pairs out.  HALF (TJ = 128): the sums of the
+// first 64 sources wait in local memory and are added to those of the second 64 before the
+// fold, so that no FP32 partial is longer than 64 terms at half the FP64 folds of tiles of 64
+// (N = 32768: 0.320 against 0.341 ms per step).  Not inlined: the loop needs every
+// register for itself (inlined into the queue loop it ran 10 % slower).
+template <int PK, int TJ, int WI, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, bool ADD,
+          bool HALF = false>
 __device__ __noinline__ bool sym_tile(const float *__restrict__ src, size_t lo_at, int n, int i0,
                                       int j0, int count, float eps2, double *acc, int at0, float *stash)
 {
@@ -348,6 +352,7 @@ __device__ __noinline__ bool sym_tile(const float *__restrict__ src, size_t lo_a
     const f2_t EPS2 = f2_pack(eps2, eps2);
     f2_t X[PK], Y[PK], Z[PK], W[PK], XL[PK], YL[PK], ZL[PK], A[PK][3];
     float ms[PK];
+    volatile f2_t first[HALF ? 3 * PK : 1];   // volatile: not in registers
 #pragma unroll
     for (int k = 0; k < PK; ++k) {
         const int i = i0 + k * 64 + 2 * lane;
@@ -454,6 +459,21 @@ __device__ __noinline__ bool sym_tile(const float *__restrict__ src, size_t lo_a
                 __syncwarp();
             }
         }
+        if (HALF && s == 32) {   // 64 sources done (count: 64 or 128)
+#pragma unroll
+            for (int k = 0; k < PK; ++k)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    first[3 * k + c] = A[k][c];
+                    A[k][c] = 0ull;
+                }
+        }
+    }
+    if (HALF) {
+#pragma unroll
+        for (int k = 0; k < PK; ++k)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) A[k][c] = f2_add(first[3 * k + c], A[k][c]);
     }
     f2_t all = 0ull;
     bool again = false;
@@ -501,20 +521,22 @@ __device__ __forceinline__ void sym_split(const float *src, size_t lo_at, int n,
 
 // One (warp, tile) by whichever of the forms above it needs.  close: BOX found
 // that it may hold close pairs.
-template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN>
+template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, bool OWN, bool HALF>
 __device__ __forceinline__ void sym_any(const float *src, size_t lo_at, int n, int i0, int j0,
                                         int count, float eps2, double *acc, float *stash, bool close)
 {
-    constexpr int WI = 64 * PK;
+    constexpr int WI = 64 * PK, LEN = HALF ? TJ / 2 : TJ;   // LEN: terms per FP32 partial
+    static_assert(!HALF || (POS == POS_SINGLE && LEN == 64), "two halves of 64 sources");
     if (!(BOX && close) &&
-        sym_tile<PK, TJ, WI, POS, BOX, WEIGHTED, KAHAN, OWN, false>(
+        sym_tile<PK, TJ, WI, POS, BOX, WEIGHTED, KAHAN, OWN, false, HALF>(
             src, lo_at, n, i0, j0, count, eps2, acc, 0, stash))
         return;
     if (POS == POS_GUARDED)
         sym_split<PK, TJ, WI, WEIGHTED, KAHAN, OWN>(src, lo_at, n, i0, j0, count, eps2, acc, stash);
     else
-        sym_slow<PK, TJ, WI, POS == POS_SPLIT, WEIGHTED, KAHAN, OWN>(src, lo_at, n, i0, j0, count, eps2,
-                                                                    acc, 0, stash, false, true);
+        for (int s = 0; s < count; s += LEN)
+            sym_slow<PK, TJ, WI, POS == POS_SPLIT, WEIGHTED, KAHAN, OWN>(
+                src, lo_at, n, i0, j0 + s, min(LEN, count - s), eps2, acc, 0, stash + s, false, true);
 }
 
 // Shared memory of each warp: its targets' accumulators and its tile's source sums.
@@ -548,7 +570,7 @@ __device__ __forceinline__ bool sym_box_close(const float4 *boxes, int t, float4
 // BOX, on spatially sorted sources: a tile whose box comes that close to the
 // box of one of the block's own tiles, and the targets' own tiles, are summed on hi/lo parts,
 // every other tile on hi parts with no test per pair.
-template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, int MINB>
+template <int PK, int TJ, int POS, bool BOX, bool WEIGHTED, bool KAHAN, int MINB, bool HALF>
 __global__ void __launch_bounds__(kSymThreads, MINB)
     force_sym_kernel(const ForceArgs p, const SymArgs q)
 {
@@ -596,10 +618,10 @@ __global__ void __launch_bounds__(kSymThreads, MINB)
                 const bool mine = j < i0 + WI;   // the sources are among the targets
                 len = min(TJ - j % TJ, it.j1 - j);
                 if (mine)
-                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, true>(
+                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, true, HALF>(
                         src, lo_at, p.n, i0, j, len, p.eps2f, acc, stash, true);
                 else
-                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, false>(
+                    sym_any<PK, TJ, POS, BOX, WEIGHTED, KAHAN, false, HALF>(
                         src, lo_at, p.n, i0, j, len, p.eps2f, acc, stash,
                         BOX && __any_sync(0xffffffffu, sym_box_close(p.boxes, j / TJ, lo, hi, rmax2,
                                                                      p.eps2f)));
