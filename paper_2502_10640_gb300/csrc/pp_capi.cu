@@ -161,7 +161,7 @@ constexpr int64_t kBoxGuardWideN = 196608;
 //   single         0.090 / 0.101 at N = 14336, 0.206 / 0.241 at 24001, 0.320 / 0.407 at
 //                  32768, 1.12 / 1.47 at 65536, 4.37 / 5.79 at 131072, 16.8 / 22.5 at 262144
 //   Kahan          0.106 / 0.099 at 14336, 0.114 / 0.117 at 15361, 0.319 / 0.452 at 32768
-//   weights        0.110 / 0.109 at 14336, 0.128 / 0.128 at 15361, 0.130 / 0.139 at 16385,
+//   weights        0.113 / 0.109 at 14336, 0.123 / 0.128 at 15361, 0.125 / 0.139 at 16385,
 //                  0.397 / 0.496 at 32768, 1.27 / 1.62 at 65536, 21.2 / 24.3 at 262144
 //   guarded        0.128 / 0.124 at 15361, 0.130 / 0.139 at 16384, 0.358 / 0.448 at 32768,
 //                  1.26 / 1.66 at 65536; on sorted sources 4.64 / 6.13 at 131072, 260 / 366
@@ -171,7 +171,8 @@ constexpr int64_t kBoxGuardWideN = 196608;
 // The tiles (64 to 512 sources) keep the FP32 partial sum of a target no longer than
 // that of the one-sided kernel that would run instead: 64 terms below N = 49152 (Kahan
 // and weights 32768, guarded 98304), 128 to 512 above.  That costs 2 % at N = 32768,
-// single (0.320 against 0.314 with 256 terms), 0 to 5 % with the blocks of 256 targets.
+// single (0.320 against 0.314 with 256 terms), 0 to 5 % with the blocks of 256 targets
+// (weights: tiles of 64 sources 2 to 4 % more than halves of 128, 24001: 0.241 / 0.231).
 // Those blocks are faster below N = 28672 (weights, 32768) and, with the test per pair,
 // at every N (guarded 65536: 1.26 against 1.30 with 512).  Above 2^22 the
 // partial sums would pass 29 GB for a step of seconds: one-sided again.
@@ -206,7 +207,7 @@ const Variant *sym_variant(const pp_ctx *c)
     }
     if (n < (c->wts || kahan ? 15361 : 14336)) return nullptr;
     if (c->wts)
-        return variant_by_name(n >= 32768 ? "f32x2w.fold64.sym8k256" : "f32x2w.fold64.sym4k64");
+        return variant_by_name(n >= 32768 ? "f32x2w.fold64.sym8k256" : "f32x2w.fold64.sym4k128h");
     if (kahan)
         return variant_by_name(n >= 32768   ? "f32x2.kahan.sym8k256"
                                : n >= 28672 ? "f32x2.kahan.sym8k64"

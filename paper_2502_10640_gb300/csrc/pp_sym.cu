@@ -57,7 +57,7 @@ std::vector<Variant> sym_variants()
         S("f32x2bguard.kahan.sym8k256", 8, 256, POS_GUARDED, false, true, 3, true),
         S("f32x2split.fold64.sym4k128", 4, 128, POS_SPLIT, false, false, 4),
         S("f32x2split.kahan.sym4k128", 4, 128, POS_SPLIT, false, true, 4),
-        S("f32x2w.fold64.sym4k64", 4, 64, POS_SINGLE, true, false, 4),
+        S("f32x2w.fold64.sym4k128h", 4, 128, POS_SINGLE, true, false, 4, false, true),
         S("f32x2w.fold64.sym8k256", 8, 256, POS_SINGLE, true, false, 2),
         S("f32x2wguard.fold64.sym4k64", 4, 64, POS_GUARDED, true, false, 4),
         S("f32x2wguard.fold64.sym4k128", 4, 128, POS_GUARDED, true, false, 4),
