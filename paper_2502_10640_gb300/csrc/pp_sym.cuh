@@ -8,7 +8,8 @@
 //
 // Decomposition.  A warp owns a block of WI = 64 PK targets (each lane PK packs
 // of two targets, positions and FP32 sums in registers) and walks a range of
-// sources at or after its block in tiles of at most TJ.  The 32 sources of a subtile sit
+// sources at or after its block in tiles of at most TJ (64 to 512: TJ is the length of
+// a target's FP32 partial sum; HALF keeps two of TJ / 2).  The 32 sources of a subtile sit
 // one per lane and rotate through the lanes by shuffle together with their
 // three sums, so after 32 steps each source has met all WI targets and is home
 // again: no cross-lane reduction, no shared-memory traffic in the loop (9
@@ -334,10 +335,10 @@ __device__ __forceinline__ void sym_collect(const ForceArgs &p, const SymArgs &q
 // place at0 of WI).  Without OWN the sources' sums go to `stash` ([3][TJ] of this
 // warp; ADD: onto what is there), every four steps, so that an FP32 partial holds
 // 8 PK terms.  OWN: the sources are among the targets; each target takes its sum
-// only (the pair comes again with the roles exchanged) and skips itself by index.  Returns false (for
-// the whole warp, nothing folded, stash void) for a tile with a zero-distance
-// pair (non-finite sum) or, with POS_GUARDED, with a pair too close for the hi
-// parts alone.  BOX: the caller has ruled close pairs out.  HALF (TJ = 128): the sums of the
+// only (the pair comes again with the roles exchanged) and skips itself by index.
+// Returns false (for the whole warp, nothing folded, stash void) for a tile with a
+// zero-distance pair (non-finite sum) or, with POS_GUARDED, with a pair too close for
+// the hi parts alone.  BOX: the caller has ruled close pairs out.  HALF (TJ = 128): the sums of the
 // first 64 sources wait in local memory and are added to those of the second 64 before the
 // fold, so that no FP32 partial is longer than 64 terms at half the FP64 folds of tiles of 64
 // (N = 32768: 0.320 against 0.341 ms per step).  Not inlined: the loop needs every

@@ -10,12 +10,12 @@
 //   s^(-3/2) = y0^3 (1 - e)^(-3/2) = y0^3 (1 + 3/2 e + 15/8 e^2 + O(e^3)),
 // whose next term is below 2^-55.  Masks (self, zero distance, padding) are
 // integer tests on the bits of s.  The one-sided kernel with the library's
-// rsqrt takes 10.4 ms per pass at N = 16385, this one 5.03.
+// rsqrt takes 10.4 ms per pass at N = 16385, this one 5.04, with the pipe 88 % busy.
 //
 // A warp owns 32 targets (one per lane, its sums in registers over a whole item)
 // and rotates 32 sources at a time through its lanes, as pp_sym.cuh does; with
 // two targets per lane the units of work are twice as long for nothing (5.36
-// against 5.03 ms per pass at N = 16385, 0.46 against 0.32 at 4096).  Two CTAs
+// against 5.04 ms per pass at N = 16385, 0.46 against 0.32 at 4096).  Two CTAs
 // per SM: the pipe needs no more than two warps per scheduler, and fewer warps
 // make the last items shorter.
 #pragma once
